@@ -1,0 +1,372 @@
+// se_fx64.cuh -- double-precision spread and gather (Eq. 3.5, Eq. 3.9 and the
+// analytic force of Sec. 3.1) in integer arithmetic.
+//
+// This GPU retires about 1.6 FP64 operations per clock and SM, but 51
+// multiply-adds of 32-bit integers into 64 bits.  The P^3 sums of a particle
+// therefore run on numbers split into two integers,
+//     v = hi + lo 2^-30,  hi = round(v), |lo| <= 2^29   (v scaled to at most 2^30),
+// whose product is  hi hi' + (hi lo' + lo hi') 2^-30  with lo lo' (below 2^-60
+// of the largest product) left out: three multiply-adds, exact, and so are
+// their sums.
+//
+//   k_scatter_fx    particles into tile order, and the window factors of each
+//                   (the only FP64 arithmetic per particle: two exponentials,
+//                   a reciprocal and two operations a factor, per dimension)
+//   k_spread_fx     Eq. 3.5: a weight is rounded to a multiple of 2^-56 max|q|
+//                   (grid_bits) and added to a 64-bit integer grid, padded so
+//                   that no support wraps, with global reductions: integer
+//                   sums, the same for every order
+//   k_fx_fold       integer grid -> FP64, its periodic images added
+//   k_grid_top, k_grid_split   largest exponent of the transformed grid, and
+//                   the grid split at that scale, padded by its periodic images
+//   k_gather_fx     Eq. 3.9 and the forces: y, x and z sums as above, one
+//                   conversion to FP64 per particle and result
+//
+// Measured against FP64 arithmetic (tiles with FP64 shared-memory adds up to P =
+// 12 and global FP64 reductions above for the spread, FP64 sums for the gather),
+// a whole evaluation: 21 642 atoms, M = 52, P = 8: 481 -> 209 us (spread 220 ->
+// 26, gather 136 -> 33); M = 96, P = 24: 2517 -> 1089 us (958 -> 396, 1324 ->
+// 446); 1000 charges, M = 32, P = 16: 181 -> 107 us (53 -> 11, 64 -> 21).  Errors
+// against 64-bit sums 3.3e-14 -> 3.5e-14 (the sums' own), 1.3e-14 -> 2.8e-15 and
+// 1.1e-15 -> 6e-16.
+//
+// Particles are taken in ranges of the tile order, so that the factors
+// (56 P bytes a particle) never need more than kFxFactorBytes.
+#pragma once
+#include <algorithm>
+
+#include "se_kernels.cuh"
+
+namespace se {
+
+// Offset of the particle from the centre of its support, as centre_offset,
+// without the rounding of x M / L (an ulp of up to M): the product enters
+// through an exact FMA and the rounding of M / L is made good.
+__device__ __forceinline__ double offset_of(double x, int c, double invh, double invh_lo) {
+    return fma(x, invh_lo, fma(x, invh, -(double)c) - 0.5);
+}
+
+__device__ __forceinline__ long long mad_wide(int a, int b, long long c) {
+    long long r;
+    asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
+    return r;
+}
+
+// The FP64 number r, |r| <= 2^30, split, by integer operations on its bits.
+__device__ __forceinline__ int2 fx_pair(double r) {
+    const long long b = __double_as_longlong(r);
+    const int sh = ((int)(b >> 52) & 0x7ff) - (1023 + 20);   // r 2^32 = mantissa 2^sh, sh <= 10
+    const long long mant = (b & 0xfffffffffffffLL) | (1LL << 52);
+    long long f = sh >= 0 ? mant << sh : (sh > -63 ? mant >> -sh : 0);
+    if (b < 0) f = -f;
+    return make_int2((int)((f + (1LL << 31)) >> 32), (int)f >> 2);
+}
+
+// 2^e (0 below the smallest subnormal), without the FP64 pipe.
+__device__ __forceinline__ double pow2i(int e) {
+    if (e >= -1022) return __hiloint2double((e + 1023) << 20, 0);
+    return e >= -1074 ? __longlong_as_double(1LL << (e + 1074)) : 0.0;
+}
+
+// Bits of the integer grid: a weight of the largest charge is below 2^bits, 56
+// but for crowded tiles, so that no grid point can reach 2^63: the weights of
+// the particles of a tile at distance d are at most e^{-beta d^2}, and summed
+// over all tiles at most crowd times the fullest tile's count (fx_params).
+__device__ __forceinline__ int grid_bits(const Acc* acc, const FxParams& fp) {
+    const int n = min(fp.kp.N, __float2int_ru(fp.crowd * (float)acc->tile_max));   // saturates
+    return min(56, 63 - (n > 1 ? 32 - __clz(n - 1) : 0));
+}
+
+// One thread per particle and dimension (dimension-major, so that a warp has
+// one).  fac[r][d][a] = (g hi, g lo, dg hi, dg lo) scaled by 2^30 and 2^(30 - sd):
+// the window and its derivative's offset factor dz g, dz = a - (P-1)/2 - u, at
+// support point a; xq[r][a] = q / max|q| times the x factor, scaled by
+// 2^(grid_bits - 27); r = position in tile order - c0.  Only particles with
+// c0 <= position < c1 get factors.  dz is split too (hi scaled by 2^26, one lo
+// for all a), so that dg costs integer operations only.
+// Bound by the FP64 pipe: two exponentials, a reciprocal and two operations a
+// factor.
+template <int P>
+__global__ void __launch_bounds__(64)
+k_scatter_fx(const double* __restrict__ xyz, const double* __restrict__ q, const FxParams fp,
+             const int* __restrict__ slot, const int* __restrict__ tile_of,
+             const int* __restrict__ tile_start, double* __restrict__ sorted,
+             int* __restrict__ perm, int* __restrict__ cells, int4* __restrict__ fac,
+             int2* __restrict__ xq, const Acc* __restrict__ acc, int c0, int c1) {
+    const KParams<double>& kp = fp.kp;
+    __shared__ double sE3[P];   // exp(-beta a_c^2) 2^30
+    if (threadIdx.x < P) sE3[threadIdx.x] = kp.E3[threadIdx.x] * 1073741824.0;
+    __syncthreads();
+    const int d = blockIdx.y;
+    const int cut = 26 + fp.sd;   // 26 to 30
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < kp.N; i += gridDim.x * blockDim.x) {
+        const int dst = tile_start[tile_of[i]] + slot[i];
+        const double x = wrap_coord(xyz[3 * (size_t)i + d], kp.L, kp.invL);
+        double s;
+        const int c = cell_of(x, kp.invh, kp.M, &s);
+        sorted[4 * (size_t)dst + d] = x;
+        cells[4 * (size_t)dst + d] = c;
+        double qp = 0.0;
+        if (d == 0) {
+            qp = q[i];
+            sorted[4 * (size_t)dst + 3] = qp;
+            perm[dst] = i;
+            qp *= acc->qscale * pow2i(grid_bits(acc, fp) - 57);
+        }
+        if (dst < c0 || dst >= c1) continue;
+        const double u = offset_of(x, c, kp.invh, fp.invh_lo);
+        // from the centre of the support outwards, so that the large factors
+        // carry the fewest roundings of the products: support points P/2 + j
+        // and P/2 - 1 - j at offsets +-(j + 1/2),
+        //   g = exp(-beta u^2 +- 2 beta u (j + 1/2)) E3
+        const double B = exp(2.0 * kp.beta * u), Bi = 1.0 / B;
+        double pu = exp(kp.beta * u * (1.0 - u)), pd = pu * Bi;
+        // dz of point P/2, in units of 2^-26
+        const double w = (0.5 - u) * 67108864.0;
+        int dzh = __double2int_rn(w);
+        const int dzl = __double2int_rn((w - (double)dzh) * 1073741824.0);
+        int4* f = fac + ((size_t)(dst - c0) * 3 + d) * P;
+        int2* xf = xq + (size_t)(dst - c0) * P;
+        auto put = [&](int a, double e, int h) {
+            const int2 g = fx_pair(e);
+            const long long cr = mad_wide(g.x, dzl, mad_wide(g.y, h, 0LL));
+            const long long v = mad_wide(g.x, h, cr >> 30);
+            const int dg = (int)((v + (1LL << (cut - 1))) >> cut);
+            f[a] = make_int4(g.x, g.y, dg, ((int)v - (int)((unsigned)dg << cut)) << (30 - cut));
+            if (d == 0) xf[a] = fx_pair(qp * e);
+        };
+#pragma unroll 2
+        for (int j = 0; j < P / 2; ++j) {
+            const int up = P / 2 + j, dn = P / 2 - 1 - j;
+            put(up, pu * sE3[up], dzh + (j << 26));
+            put(dn, pd * sE3[dn], dzh - ((j + 1) << 26));
+            pu *= B;
+            pd *= Bi;
+        }
+    }
+}
+
+// Particles of a warp: a lane per z point.
+template <int P>
+constexpr int kFxGPW = 32 / P;
+// rows of the support whose factors a lane of the spread keeps in registers
+template <int P>
+constexpr int kFxRows = P <= 16 ? P : P / 2;
+// rows of the support whose grid values a lane loads at once
+template <int P>
+constexpr int kFxBatch = P <= 12 ? P : (P % 8 == 0 ? 8 : P / 2);
+constexpr int kFxThreads = 128;
+
+// Spread.  The integer grid is padded as the split one (k_gather_fx).  A lane
+// holds its z point's factor times the y factors (kFxRows rows at a time) and
+// runs over the x planes; the weight xq yz is
+//   W = xhi yzhi + (xhi yzlo + xlo yzhi) 2^-30,  |W| < 2^59,
+// an integer in units of 2^-3 of the grid's.  Particles come in tile order, but
+// nothing depends on it.
+// Bound by the L2's 64-bit reductions (about 2.4 lanes per clock and SM).
+template <int P>
+__global__ void __launch_bounds__(kFxThreads)
+k_spread_fx(const int4* __restrict__ fac, const int2* __restrict__ xq,
+            const int* __restrict__ cells, unsigned long long* __restrict__ g64, int Mp, int c0,
+            int c1) {
+    constexpr int GPW = kFxGPW<P>, BC = kFxRows<P>;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int gi = lane / P, k = lane - gi * P;
+    if (gi >= GPW) return;
+    const int per = (kFxThreads / 32) * GPW;
+    for (long long pl = c0 + (long long)blockIdx.x * per + warp * GPW + gi; pl < c1;
+         pl += (long long)gridDim.x * per) {
+        const int p = (int)pl;
+        const int4 cell = *reinterpret_cast<const int4*>(cells + 4 * (size_t)p);
+        const int4* fy = fac + ((size_t)(p - c0) * 3 + 1) * P;
+        const int2* fx = xq + (size_t)(p - c0) * P;
+        const int2 z = *reinterpret_cast<const int2*>(fy + P + k);
+        unsigned long long* g0 = g64 + ((size_t)cell.x * Mp + cell.y) * Mp + cell.z + k;
+#pragma unroll 1
+        for (int bc = 0; bc < P; bc += BC) {
+            int yzh[BC], yzl[BC];
+#pragma unroll
+            for (int b = 0; b < BC; ++b) {
+                const int2 y = __ldg(reinterpret_cast<const int2*>(fy + bc + b));
+                const long long cr = mad_wide(y.x, z.y, mad_wide(y.y, z.x, 0LL));
+                const long long v = mad_wide(y.x, z.x, cr >> 30);
+                yzh[b] = (int)((v + (1 << 29)) >> 30);
+                yzl[b] = (int)v - (int)((unsigned)yzh[b] << 30);
+            }
+            unsigned long long* ga = g0 + (size_t)bc * Mp;
+#pragma unroll 1
+            for (int a = 0; a < P; ++a, ga += (size_t)Mp * Mp) {
+                const int2 x = __ldg(fx + a);
+                unsigned long long* g = ga;
+#pragma unroll
+                for (int b = 0; b < BC; ++b, g += Mp) {
+                    // + 4: the cut of three bits rounds
+                    const long long cr = mad_wide(x.x, yzl[b], mad_wide(x.y, yzh[b], 4LL << 30));
+                    const long long w = mad_wide(x.x, yzh[b], (long long)(int)(cr >> 30));
+                    atomicAdd(g, (unsigned long long)(w >> 3));
+                }
+            }
+        }
+    }
+}
+
+// A sum of products of split numbers: A + B 2^-30.
+struct FxSum {
+    long long A, B;
+    __device__ __forceinline__ void mac(int2 h, int2 g) {
+        A = mad_wide(g.x, h.x, A);
+        B = mad_wide(g.x, h.y, B);
+        B = mad_wide(g.y, h.x, B);
+    }
+    __device__ __forceinline__ long long value() const { return A + (B >> 30); }
+};
+// The sum times 2^-(32 + e), split.
+__device__ __forceinline__ int2 fx_top(const FxSum& s, int e) {
+    const long long v = s.value() >> e;
+    return make_int2((int)((v + (1LL << 31)) >> 32), (int)v >> 2);
+}
+
+// Gather (Eq. 3.9, Sec. 3.1): one lane per z point sums over y, then x, as in
+// gather_accum, then the lanes' sums are multiplied by the z factors and added
+// over the lanes.  The grid is split and padded (k_grid_split): support point
+// (a, b, c) of a particle in cell (cx, cy, cz) is grid[(cx + a) Mp + cy + b) Mp +
+// cz + c], Mp = M + P - 1, so that the rows of the support are a constant apart.
+// Particles come in tile order, so that the L1 cache serves most of the loads.
+// Scales: the grid's hi has hb bits (30 for all but the flattest windows), and
+// each of the three sums is at most gs times the largest term, gs a bound of
+// the sum of a window's factors; the first two are cut to 32 + e1 and 32 + e2
+// bits less, so that every sum stays below 2^63 (fx_params).
+// Bound by the integer multiply-adds: six of about nine instructions a grid
+// value for potential and force.
+// Consecutive particles share a block, and with it the L1 cache: up to 512
+// threads (fewer where the particles are too few for every SM).  Supports 14 and
+// 16 keep 16 rows of loads and factors in flight in more than 128 registers
+// (P = 16, 1000 charges: 21 us against 37 at 128).
+template <int P>
+__global__ void __launch_bounds__(P <= 16 ? 256 : 512, P == 14 || P == 16 ? 1 : 2)
+k_gather_fx(const int4* __restrict__ fac, const int* __restrict__ cells,
+            const double* __restrict__ sorted, const int* __restrict__ perm,
+            const int2* __restrict__ grid, const unsigned* __restrict__ top,
+            double* __restrict__ phi, double* __restrict__ F, const FxParams fp,
+            double* __restrict__ parts, unsigned* ticket, Acc* acc, double e_scale, double* E_out,
+            const double* __restrict__ adj, int c0, int c1) {
+    constexpr int GPW = kFxGPW<P>, UB = kFxBatch<P>;
+    constexpr bool kHold = P <= 12;   // y factors in registers, else loaded again for each x
+    const KParams<double>& kp = fp.kp;
+    __shared__ double sbuf[32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int gi = lane / P, k = lane - gi * P;
+    const int Mp = kp.M + P - 1;
+    // the grid's units 2^(E - hb); the sums are scaled by 2^30 per window and
+    // cut by 2^(32 + e1) and 2^(32 + e2)
+    const double unit = pow2i((int)top[0] - 1022 - fp.hb - 26 + fp.e1 + fp.e2);
+    const double gsc = adj ? __ldg(adj) : 1.0;
+    const double u_phi = unit * kp.phi_scale;
+    const double u_F = unit * kp.F_scale * pow2i(fp.sd) * (adj ? -gsc : 1.0);
+    double e_loc = 0.0;
+    const int per = (blockDim.x >> 5) * GPW;
+    for (long long pb = c0 + (long long)blockIdx.x * per + warp * GPW; pb < c1;
+         pb += (long long)gridDim.x * per) {
+        const int p = (int)pb + gi;
+        const bool valid = gi < GPW && p < c1;
+        long long v[4] = {0, 0, 0, 0};
+        if (valid) {
+            const int4* f = fac + (size_t)(p - c0) * 3 * P;
+            const int4 cell = *reinterpret_cast<const int4*>(cells + 4 * (size_t)p);
+            const int2* row0 = grid + ((size_t)cell.x * Mp + cell.y) * Mp + cell.z + k;
+            int2 g[kHold ? P : 1], dg[kHold ? P : 1];
+            if constexpr (kHold) {
+#pragma unroll
+                for (int b = 0; b < P; ++b) {
+                    const int4 y = __ldg(f + P + b);
+                    g[b] = make_int2(y.x, y.y);
+                    dg[b] = make_int2(y.z, y.w);
+                }
+            }
+            FxSum s0 = {0, 0}, sx = {0, 0}, sy = {0, 0};
+#pragma unroll 1
+            for (int a = 0; a < P; ++a) {
+                const int4 xa = __ldg(f + a);
+                const int2* row = row0;
+                row0 += (size_t)Mp * Mp;
+                FxSum t0 = {0, 0}, t1 = {0, 0};
+#pragma unroll
+                for (int b0 = 0; b0 < P; b0 += UB) {
+                    int2 w[UB];
+#pragma unroll
+                    for (int b = 0; b < UB; ++b, row += Mp) w[b] = __ldg(row);
+#pragma unroll
+                    for (int b = 0; b < UB; ++b) {
+                        if constexpr (kHold) {
+                            t0.mac(w[b], g[b]);
+                            t1.mac(w[b], dg[b]);
+                        } else {
+                            const int4 y = __ldg(f + P + b0 + b);
+                            t0.mac(w[b], make_int2(y.x, y.y));
+                            t1.mac(w[b], make_int2(y.z, y.w));
+                        }
+                    }
+                }
+                const int2 gx = make_int2(xa.x, xa.y), dgx = make_int2(xa.z, xa.w);
+                const int2 n0 = fx_top(t0, fp.e1), n1 = fx_top(t1, fp.e1);
+                s0.mac(n0, gx);
+                sx.mac(n0, dgx);
+                sy.mac(n1, gx);
+            }
+            // z: the lane's share of the four results
+            const int4 za = __ldg(f + 2 * P + k);
+            const int2 gz = make_int2(za.x, za.y), dgz = make_int2(za.z, za.w);
+            const int2 n0 = fx_top(s0, fp.e2), nx = fx_top(sx, fp.e2), ny = fx_top(sy, fp.e2);
+            FxSum t[4] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};
+            t[0].mac(n0, gz);
+            t[1].mac(nx, gz);
+            t[2].mac(ny, gz);
+            t[3].mac(n0, dgz);
+#pragma unroll
+            for (int c = 0; c < 4; ++c) v[c] = t[c].value();
+        }
+#pragma unroll
+        for (int o = 1; o < P; o <<= 1) {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const long long a = __shfl_down_sync(0xffffffffu, v[c], o);
+                if (k + o < P) v[c] += a;
+            }
+        }
+        // result c to lane c of the group: one conversion and two products a lane
+        long long mine[(4 + P - 1) / P];
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const long long t = __shfl_sync(0xffffffffu, v[c], lane - k);
+            if (k == c % P) mine[c / P] = t;
+        }
+        if (valid) {
+            const double qq = sorted[4 * (size_t)p + 3];
+            const int orig = perm[p];
+#pragma unroll
+            for (int j = 0; j < (4 + P - 1) / P; ++j) {
+                const int c = k + j * P;
+                if (c > 3) break;
+                const double w = (double)mine[j] * (c == 0 ? u_phi : u_F);
+                if (c == 0) {
+                    if (phi) phi[orig] = w * gsc;
+                    e_loc += qq * w;
+                } else if (F) {
+                    F[3 * (size_t)orig + c - 1] = w * qq;
+                }
+            }
+        }
+    }
+    const double r = block_sum(e_loc, sbuf);
+    if (threadIdx.x == 0) parts[blockIdx.x] = r;
+    if (!last_block(ticket)) return;
+    const double s = sum_partials(parts, gridDim.x, 1, 0, sbuf);
+    if (threadIdx.x == 0) {
+        const double e = c0 == 0 ? s : acc->e_gather + s;   // later ranges add to the first
+        acc->e_gather = e;
+        if (E_out) *E_out = e_scale * e;
+        *ticket = 0u;
+    }
+}
+
+}  // namespace se

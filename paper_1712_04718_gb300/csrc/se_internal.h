@@ -44,7 +44,9 @@ struct Acc {
     unsigned int nonfinite;  // number of particles with NaN/Inf position or charge (bin)
     int fx_shift;            // fixed-point spread: weights scaled by 2^fx_shift
     float fx_scale, fx_inv;  // 2^fx_shift and 2^-fx_shift
-    double pad;
+    double qscale, qunit;    // 1 / max|q| (a little less) and its inverse (k_bin)
+    int tile_max;            // particles of the fullest tile (k_bin)
+    int pad;
 };
 
 // launchers (se_kernels_*.cu)
@@ -87,6 +89,41 @@ cudaError_t launch_gather_plain(int ng, const v4_t<T>* sorted, const int* perm, 
                                 size_t gstride, T* phi, T* F, const KParams<T>& kp,
                                 double* partials, unsigned* ticket, Acc* acc, double e_scale,
                                 double* E_out, bool pdl, cudaStream_t s);
+
+// Double-precision spread and gather in integer arithmetic (se_fx64.cuh).
+struct FxParams {
+    KParams<double> kp;
+    double invh_lo;   // M / L - kp.invh, to FP64 accuracy
+    int sd;           // 2^sd bounds the derivative window's factors
+    int hb;           // integer bits of the split grid
+    float crowd;      // see grid_bits
+    int e1, e2;       // the gather's sums over y and x are cut by 32 + e1, 32 + e2 bits
+};
+constexpr size_t kFxFactorBytes = (size_t)4 << 30;   // window factors of one range of particles
+constexpr int kFxTopBlocks = 512;
+struct FxBufs {
+    long long* g64;        // (M + P - 1)^3: the integer grid, zero between calls
+    double* grid;          // M^3: the FP64 spread grid
+    void* fac;             // int4 [cap][3][P] window factors
+    void* xq;              // int2 [cap][P] charge times x factors
+    int cap;               // particles of a range
+    int* cells;            // int4 [N]: cells of the particles in tile order
+    int *slot, *tile_of, *tile_start, *perm;
+    void* sorted;          // d4 [N]
+    void* split;           // int2 [(M + P - 1)^3]: the transformed grid, split and padded
+    unsigned* top;         // [kFxTopBlocks]: per-block largest high words, then the exponent
+    double* parts;         // [nparts] energy partials
+    int nparts;
+    unsigned* ticket;
+    Acc* acc;
+};
+// after launch_bin<double>: factors, spread, FP64 grid; mark(ctx, 1) after the scatter
+// (with `only` the particles in tile order and the factors, no spread)
+cudaError_t fx_spread(const double* xyz, const double* q, const FxParams& fp, const FxBufs& b,
+                      bool only, cudaStream_t s, void (*mark)(void*, int), void* ctx);
+cudaError_t fx_gather(const double* xyz, const double* q, const FxParams& fp, const FxBufs& b,
+                      const double* grid, double* phi, double* F, double e_scale, double* E_out,
+                      const double* adj, cudaStream_t s);
 
 // Kernel parameters for an FP64 evaluation without a plan (se_plan.cu).
 int make_kparams_f64(int64_t N, double L, double xi, int M, int P, int tile, KParams<double>* out);

@@ -233,18 +233,19 @@ __device__ __forceinline__ df2 warp_sum_partials_df(const float* partials, int n
 
 // Last-block detection: every block stores its partial, fences, and takes a
 // ticket; the block with the last ticket sees all partials.
-__device__ __forceinline__ bool last_block(unsigned* ticket) {
+__device__ __forceinline__ bool last_block2(unsigned* ticket, unsigned nblocks) {
     __shared__ bool is_last;
     __threadfence();
     __syncthreads();
     if (threadIdx.x == 0) {
         unsigned t = atomicAdd(ticket, 1u);
-        is_last = (t == gridDim.x - 1);
+        is_last = (t == nblocks - 1);
     }
     __syncthreads();
     if (is_last) __threadfence();
     return is_last;
 }
+__device__ __forceinline__ bool last_block(unsigned* ticket) { return last_block2(ticket, gridDim.x); }
 
 // Sum of n partials (stride apart, from offset), by the whole block; valid in
 // thread 0.  The loads go through L2 (other blocks wrote them).
@@ -264,10 +265,17 @@ template <typename T>
 __global__ void __launch_bounds__(256)
 k_bin(const T* __restrict__ xyz, const T* __restrict__ q, const KParams<T> kp,
       int* __restrict__ tile_count, int* __restrict__ slot, int* __restrict__ tile_of,
-      int* __restrict__ tile_start, double* __restrict__ partials, unsigned* ticket,
-      Acc* acc) {
+      int* __restrict__ tile_start, double* __restrict__ partials,
+      unsigned long long* __restrict__ qmax_part, unsigned* ticket, Acc* acc) {
     __shared__ double sbuf[32];
+    __shared__ unsigned long long sqm;
+    __shared__ int s_tmax;
     double sq = 0.0, sa = 0.0, bad = 0.0;
+    unsigned long long qm = 0u;   // bits of the largest finite |q| (as a double)
+    if (threadIdx.x == 0) {
+        sqm = 0u;
+        s_tmax = 0;
+    }
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < kp.N; i += gridDim.x * blockDim.x) {
         T x = xyz[3 * i], y = xyz[3 * i + 1], z = xyz[3 * i + 2], qq = q[i];
         if (!(isfinite(x) && isfinite(y) && isfinite(z) && isfinite(qq))) bad += 1.0;
@@ -280,16 +288,39 @@ k_bin(const T* __restrict__ xyz, const T* __restrict__ q, const KParams<T> kp,
         tile_of[i] = tile;
         sq += (double)qq;
         sa += fabs((double)qq);
+        const unsigned long long b = (unsigned long long)__double_as_longlong(fabs((double)qq));
+        if (b < 0x7ff0000000000000ull && b > qm) qm = b;
     }
     double r0 = block_sum(sq, sbuf);
     double r1 = block_sum(sa, sbuf);
     double r2 = block_sum(bad, sbuf);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long v = __shfl_xor_sync(0xffffffffu, qm, o);
+        qm = v > qm ? v : qm;
+    }
+    if ((threadIdx.x & 31) == 0) atomicMax(&sqm, qm);
+    __syncthreads();
     if (threadIdx.x == 0) {
         partials[3 * blockIdx.x] = r0;
         partials[3 * blockIdx.x + 1] = r1;
         partials[3 * blockIdx.x + 2] = r2;
+        qmax_part[blockIdx.x] = sqm;
     }
     if (!last_block(ticket)) return;
+    if (threadIdx.x == 0) sqm = 0u;
+    __syncthreads();
+    qm = 0u;
+    for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) {
+        const unsigned long long v = __ldcg(qmax_part + b);
+        qm = v > qm ? v : qm;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const unsigned long long v = __shfl_xor_sync(0xffffffffu, qm, o);
+        qm = v > qm ? v : qm;
+    }
+    if ((threadIdx.x & 31) == 0) atomicMax(&sqm, qm);
 
     // --- last block: checks, exclusive scan of the tile counts ---
     {
@@ -300,6 +331,10 @@ k_bin(const T* __restrict__ xyz, const T* __restrict__ q, const KParams<T> kp,
             acc->sum_q = a;
             acc->sum_absq = b;
             acc->nonfinite = (unsigned)c;
+            // the scale of the charges: |q| qscale < 1; charges below 2^-1000 keep 2^1000
+            const double qmax = __longlong_as_double((long long)sqm);
+            acc->qscale = qmax > 0x1p-1000 ? (1.0 - 0x1p-50) / qmax : 0x1p+1000;
+            acc->qunit = 1.0 / acc->qscale;
             *ticket = 0u;
         }
     }
@@ -315,7 +350,13 @@ k_bin(const T* __restrict__ xyz, const T* __restrict__ q, const KParams<T> kp,
     const int per = (n + blockDim.x - 1) / blockDim.x;
     const int b0 = min(n, (int)threadIdx.x * per), b1 = min(n, b0 + per);
     int local = 0;
-    for (int k = b0; k < b1; ++k) local += staged ? scount[k] : __ldcg(tile_count + k);
+    int tmax = 0;
+    for (int k = b0; k < b1; ++k) {
+        const int cnt = staged ? scount[k] : __ldcg(tile_count + k);
+        local += cnt;
+        tmax = max(tmax, cnt);
+    }
+    atomicMax(&s_tmax, tmax);
     // block exclusive scan of `local`
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int incl = local;
@@ -344,7 +385,10 @@ k_bin(const T* __restrict__ xyz, const T* __restrict__ q, const KParams<T> kp,
         run += cnt;
     }
     for (int k = threadIdx.x; k < n; k += blockDim.x) tile_count[k] = 0;
-    if (threadIdx.x == blockDim.x - 1) tile_start[n] = run;
+    if (threadIdx.x == blockDim.x - 1) {
+        tile_start[n] = run;
+        acc->tile_max = s_tmax;
+    }
 }
 
 // a1: scatter into tile order: sorted[tile_start[tile] + slot] = (x, y, z, q).

@@ -2,4 +2,5 @@
 #include "se_launch.cuh"
 namespace se {
 SE_INSTANTIATE(float)
+SE_INSTANTIATE_GATHER(float)
 }

@@ -21,7 +21,9 @@ cudaError_t launch_bin(const T* xyz, const T* q, const KParams<T>& kp, int* tile
                        unsigned* ticket, Acc* acc, cudaStream_t s) {
     int blocks = std::max(1, std::min((kp.N + kThreads - 1) / kThreads, kMaxPartials));
     k_bin<T><<<blocks, kThreads, 0, s>>>(xyz, q, kp, tile_count, slot, tile_of, tile_start,
-                                         partials, ticket, acc);
+                                         partials,
+                                         reinterpret_cast<unsigned long long*>(partials + 3 * kMaxPartials),
+                                         ticket, acc);
     return cudaGetLastError();
 }
 
@@ -135,7 +137,8 @@ cudaError_t launch_gather(const v4_t<T>* sorted, const int* perm, const T* grid,
     template cudaError_t launch_spread_direct<T>(const v4_t<T>*, T*, const KParams<T>&,         \
                                                  cudaStream_t);                                 \
     template cudaError_t launch_scale<T>(void*, const double*, int, T*, double*, unsigned*,     \
-                                         Acc*, double, double*, cudaStream_t);                  \
+                                         Acc*, double, double*, cudaStream_t);
+#define SE_INSTANTIATE_GATHER(T)                                                                \
     template cudaError_t launch_gather<T>(const v4_t<T>*, const int*, const T*, T*, T*,         \
                                           const KParams<T>&, double*, unsigned*, Acc*, double,  \
                                           double*, const double*, cudaStream_t);

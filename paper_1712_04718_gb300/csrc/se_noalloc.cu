@@ -37,7 +37,7 @@ constexpr size_t kOffTileOf = up256(kOffSlot + sizeof(int) * kNoAllocMaxN);
 constexpr size_t kOffPerm = up256(kOffTileOf + sizeof(int) * kNoAllocMaxN);
 constexpr size_t kOffSorted = up256(kOffPerm + sizeof(int) * kNoAllocMaxN);
 constexpr size_t kOffPartials = up256(kOffSorted + sizeof(se::d4) * kNoAllocMaxN);
-constexpr size_t kOffTickets = up256(kOffPartials + sizeof(double) * 3 * se::kMaxPartials);
+constexpr size_t kOffTickets = up256(kOffPartials + sizeof(double) * 4 * se::kMaxPartials);
 constexpr size_t kOffAcc = up256(kOffTickets + sizeof(unsigned) * 4);
 constexpr size_t kScratchBytes = up256(kOffAcc + sizeof(se::Acc));
 

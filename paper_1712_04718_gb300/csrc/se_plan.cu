@@ -79,6 +79,18 @@ struct se_plan {
     unsigned* tickets = nullptr;   // 8 counters (see FastBufs)
     Acc* acc = nullptr;
     double* dE = nullptr;          // device energy for se_energy_force
+    // double precision, analytic forces: window factors of fx_cap particles
+    // (se_fx64.cuh), cells in tile order, the split grid's exponent, energy
+    // partials of the tiles
+    void* fx_fac = nullptr;
+    void* fx_xq = nullptr;
+    int fx_cap = 0;
+    int* fx_cells = nullptr;
+    unsigned* fx_top = nullptr;
+    void* fx_split = nullptr;
+    void* fx_grid = nullptr;
+    double* fx_parts = nullptr;
+    int fx_nparts = 0;
     cufftHandle fwd = 0, inv = 0;
     bool have_fft = false;
     // staging buffers of se_energy_force_host
@@ -199,7 +211,7 @@ void derive(se_plan* p) {
     // ik forces need the three extra inverse transforms of the cuFFT pipeline
     if (p->force_mode == SE_FORCE_IK && variant >= 3) variant = 0;
     if (variant == 0) {
-        if (p->prec == SE_FP64) variant = p->P > 12 ? 2 : 1;
+        if (p->prec == SE_FP64) variant = 1;
         else variant = (fast_ok && p->force_mode != SE_FORCE_IK) ? 3 : 1;
     }
     if (p->prec == SE_FP32 && variant == 2) variant = 1;  // the compensated sum needs the tiles
@@ -233,13 +245,19 @@ void release_device(se_plan* p) {
     void* bufs[] = {p->grid_spread, p->grid_gather, p->cgrid, p->green, p->tile_count,
                     p->tile_start, p->slot, p->tile_of, p->perm, p->sorted, p->partials,
                     p->tickets, p->acc, p->dE, p->h_xyz, p->h_q, p->h_F, p->h_phi, p->g64, p->tw, p->green_f,
-                    p->bucket, p->bucket_idx, p->cgrid_ik, p->part};
+                    p->bucket, p->bucket_idx, p->cgrid_ik, p->part, p->fx_fac, p->fx_xq,
+                    p->fx_cells, p->fx_top, p->fx_split, p->fx_grid, p->fx_parts};
     for (void* b : bufs)
         if (b) cudaFree(b);
     p->grid_spread = p->grid_gather = p->cgrid = p->sorted = p->tw = p->bucket = nullptr;
     p->bucket_idx = nullptr;
     p->cgrid_ik = nullptr;
     p->part = nullptr;
+    p->fx_fac = p->fx_xq = nullptr;
+    p->fx_cells = nullptr;
+    p->fx_top = nullptr;
+    p->fx_split = p->fx_grid = nullptr;
+    p->fx_parts = nullptr;
     p->g64 = nullptr;
     p->green_f = nullptr;
     p->green = p->partials = p->dE = nullptr;
@@ -348,6 +366,21 @@ int prepare(se_plan* p) {
     if (rc == SE_OK) rc = dalloc((void**)&p->tickets, 8 * sizeof(unsigned));
     if (rc == SE_OK) rc = dalloc((void**)&p->acc, sizeof(Acc));
     if (rc == SE_OK) rc = dalloc((void**)&p->dE, sizeof(double));
+    if (p->prec == SE_FP64) {
+        const size_t per = (size_t)56 * p->P;   // bytes of factors a particle
+        p->fx_cap = (int)std::max<size_t>(1, std::min(N, se::kFxFactorBytes / per));
+        if (rc == SE_OK) rc = dalloc(&p->fx_fac, (size_t)p->fx_cap * 48 * p->P);
+        if (rc == SE_OK) rc = dalloc(&p->fx_xq, (size_t)p->fx_cap * 8 * p->P);
+        if (rc == SE_OK) rc = dalloc((void**)&p->fx_cells, N * 4 * sizeof(int));
+        if (rc == SE_OK) rc = dalloc((void**)&p->fx_top, (se::kFxTopBlocks + 1) * sizeof(unsigned));
+        const size_t Mp = (size_t)p->M + p->P - 1;
+        if (rc == SE_OK) rc = dalloc(&p->fx_split, Mp * Mp * Mp * 2 * sizeof(int));
+        if (rc == SE_OK) rc = dalloc(&p->fx_grid, Mp * Mp * Mp * sizeof(long long));
+        if (rc == SE_OK && cudaMemset(p->fx_grid, 0, Mp * Mp * Mp * sizeof(long long)) != cudaSuccess)
+            rc = SE_ERR_CUDA;
+        p->fx_nparts = (int)std::min<size_t>(1 << 16, N + 1);
+        if (rc == SE_OK) rc = dalloc((void**)&p->fx_parts, (size_t)p->fx_nparts * sizeof(double));
+    }
     if (rc != SE_OK) {
         release_device(p);
         return rc;
@@ -440,6 +473,57 @@ se::FastBufs fast_bufs(se_plan* p) {
     return b;
 }
 
+// Scales of the double-precision integer gather (se_fx64.cuh): bounds of a
+// window's factors g = e^{-beta x^2} and |x| g at P points one apart, by
+// integral plus maximum (twice the maximum for the two-peaked one).
+se::FxParams fx_params(const se_plan* p) {
+    se::FxParams f;
+    f.kp = make_kparams<double>(p);
+    const long double invh = (long double)p->M / (long double)p->L;
+    f.invh_lo = (double)(invh - (long double)f.kp.invh);
+    const double beta = f.kp.beta, P = p->P;
+    const double dmax = std::min(0.5 * P, exp(-0.5) / sqrt(2.0 * beta));
+    f.sd = std::max(0, (int)ceil(log2(dmax)));
+    const double g = std::min(P, sqrt(kPi / beta) + 1.0);
+    const double dg = std::min(P * dmax, 1.0 / beta + 2.0 * dmax) * ldexp(1.0, -f.sd);
+    // the sums over y, x and z in bits, each kept below 63 (a margin of 2^-6
+    // covers the rounding of the factors and of the bound)
+    const double gs = log2(std::max(g, dg)) + 1.0 / 64.0, top = 63.0;
+    // the tiles' largest weights at a point, summed over the tiles: at a face,
+    // distances 0, 0, T, T, 2T, 2T, ... per dimension
+    double k = 0.0;
+    for (int i = 0; i * p->tile <= p->P; ++i) k += 2.0 * exp(-beta * i * p->tile * i * p->tile);
+    f.crowd = (float)(k * k * k * (1.0 + 1e-6));
+    f.hb = std::min(30, (int)floor(top - 30.0 - gs));
+    const double s1 = 30.0 + f.hb + gs;                              // sum over y
+    f.e1 = std::max(0, (int)ceil(30.0 + gs + s1 - 32.0 - top));
+    const double s2 = 30.0 + gs + s1 - 32.0 - f.e1;                  // sum over x
+    f.e2 = std::max(0, (int)ceil(30.0 + gs + s2 - 32.0 - top));
+    return f;
+}
+
+se::FxBufs fx_bufs(se_plan* p) {
+    se::FxBufs b;
+    b.g64 = (long long*)p->fx_grid;
+    b.grid = (double*)p->grid_spread;
+    b.fac = p->fx_fac;
+    b.xq = p->fx_xq;
+    b.cap = p->fx_cap;
+    b.cells = p->fx_cells;
+    b.slot = p->slot;
+    b.tile_of = p->tile_of;
+    b.tile_start = p->tile_start;
+    b.perm = p->perm;
+    b.sorted = p->sorted;
+    b.split = p->fx_split;
+    b.top = p->fx_top;
+    b.parts = p->fx_parts;
+    b.nparts = p->fx_nparts;
+    b.ticket = p->tickets + 2;
+    b.acc = p->acc;
+    return b;
+}
+
 void mark_cb(void* ctx, int s) { timing_mark(static_cast<se_plan*>(ctx), s); }
 
 
@@ -513,20 +597,32 @@ int do_spread(se_plan* p, const void* xyz, const void* q) {
     const KParams<T> kp = make_kparams<T>(p);
     using V = se::v4_t<T>;
     const size_t M3 = (size_t)p->M * p->M * p->M;
-    if (!p->spread_clean) SE_CUDA(cudaMemsetAsync(p->grid_spread, 0, M3 * sizeof(T), p->stream));
+    // the integer spread overwrites the FP64 grid; the others add to it
+    const bool adds = std::is_same<T, float>::value || p->variant == 2;
+    if (adds && !p->spread_clean)
+        SE_CUDA(cudaMemsetAsync(p->grid_spread, 0, M3 * sizeof(T), p->stream));
     timing_begin(p);
     SE_CUDA(se::launch_bin<T>((const T*)xyz, (const T*)q, kp, p->tile_count, p->slot, p->tile_of,
                               p->tile_start, p->partials, p->tickets + 0, p->acc, p->stream));
     timing_mark(p, 0);
-    SE_CUDA(se::launch_scatter<T>((const T*)xyz, (const T*)q, kp, p->slot, p->tile_of,
-                                  p->tile_start, (V*)p->sorted, p->perm, p->stream));
-    timing_mark(p, 1);
-    if (p->N > 0) {
-        if (p->variant == 2)
+    if constexpr (std::is_same<T, double>::value) {
+        // factors (for the gather too), then the spread; variant 2 spreads with
+        // global FP64 reductions instead
+        SE_CUDA(se::fx_spread((const double*)xyz, (const double*)q, fx_params(p), fx_bufs(p),
+                              p->variant == 2, p->stream, mark_cb, p));
+        if (p->N > 0 && p->variant == 2)
             SE_CUDA(se::launch_spread_direct<T>((const V*)p->sorted, (T*)p->grid_spread, kp, p->stream));
-        else
-            SE_CUDA(se::launch_spread_tiled<T>((const V*)p->sorted, p->tile_start, (T*)p->grid_spread,
-                                               kp, p->prec == SE_FP32, p->stream));
+    } else {
+        SE_CUDA(se::launch_scatter<T>((const T*)xyz, (const T*)q, kp, p->slot, p->tile_of,
+                                      p->tile_start, (V*)p->sorted, p->perm, p->stream));
+        timing_mark(p, 1);
+        if (p->N > 0) {
+            if (p->variant == 2)
+                SE_CUDA(se::launch_spread_direct<T>((const V*)p->sorted, (T*)p->grid_spread, kp, p->stream));
+            else
+                SE_CUDA(se::launch_spread_tiled<T>((const V*)p->sorted, p->tile_start, (T*)p->grid_spread,
+                                                   kp, p->prec == SE_FP32, p->stream));
+        }
     }
     timing_mark(p, 2);
     p->spread_clean = false;
@@ -547,13 +643,15 @@ int do_scale(se_plan* p, double* E_grid) {
     const double M3 = (double)p->M * p->M * p->M;
     const double e_scale = p->kc * p->h * p->h * p->h / (2.0 * M3);
     const bool ik = p->force_mode == SE_FORCE_IK;
+    // cleared for the next spread, unless that overwrites it
+    T* zero = std::is_same<T, float>::value || p->variant == 2 ? (T*)p->grid_spread : nullptr;
     if (ik)
         SE_CUDA(se::launch_scale_ik<T>(p->cgrid, p->cgrid_ik, ik_cstride(p), p->green, p->M, p->L,
-                                       (T*)p->grid_spread,
+                                       zero,
                                        p->partials + 3 * se::kMaxPartials, p->tickets + 1, p->acc,
                                        e_scale, E_grid, p->stream));
     else
-        SE_CUDA(se::launch_scale<T>(p->cgrid, p->green, p->M, (T*)p->grid_spread, p->partials + 3 * se::kMaxPartials,
+        SE_CUDA(se::launch_scale<T>(p->cgrid, p->green, p->M, zero, p->partials + 3 * se::kMaxPartials,
                                     p->tickets + 1, p->acc, e_scale, E_grid, p->stream));
     timing_mark(p, 4);
     p->spread_clean = true;
@@ -575,7 +673,8 @@ int do_scale(se_plan* p, double* E_grid) {
 }
 
 template <typename T>
-int do_gather(se_plan* p, void* phi, void* F, double* E, const double* adj = nullptr) {
+int do_gather(se_plan* p, const void* xyz, const void* q, void* phi, void* F, double* E,
+              const double* adj = nullptr) {
     const KParams<T> kp = make_kparams<T>(p);
     using V = se::v4_t<T>;
     // ik forces: potential and force from the four grids with the plain window;
@@ -587,6 +686,9 @@ int do_gather(se_plan* p, void* phi, void* F, double* E, const double* adj = nul
                                            ik_gstride(p), (T*)phi, (T*)F, kp,
                                            p->partials + 4 * se::kMaxPartials, p->tickets + 2,
                                            p->acc, 0.5, E, false, p->stream));
+    else if constexpr (std::is_same<T, double>::value)
+        SE_CUDA(se::fx_gather((const T*)xyz, (const T*)q, fx_params(p), fx_bufs(p),
+                              (const T*)p->grid_gather, (T*)phi, (T*)F, 0.5, E, adj, p->stream));
     else
         SE_CUDA(se::launch_gather<T>((const V*)p->sorted, p->perm, (const T*)p->grid_gather, (T*)phi,
                                      (T*)F, kp, p->partials + 4 * se::kMaxPartials, p->tickets + 2,
@@ -622,11 +724,11 @@ int evaluate(se_plan* p, const void* xyz, const void* q, void* F, void* phi, dou
     if (p->prec == SE_FP64) {
         SE_TRY(do_spread<double>(p, xyz, q));
         SE_TRY(do_scale<double>(p, energy_only ? dE : nullptr));
-        if (!energy_only) SE_TRY(do_gather<double>(p, phi, F, dE));
+        if (!energy_only) SE_TRY(do_gather<double>(p, xyz, q, phi, F, dE));
     } else {
         SE_TRY(do_spread<float>(p, xyz, q));
         SE_TRY(do_scale<float>(p, energy_only ? dE : nullptr));
-        if (!energy_only) SE_TRY(do_gather<float>(p, phi, F, dE));
+        if (!energy_only) SE_TRY(do_gather<float>(p, xyz, q, phi, F, dE));
     }
     return SE_OK;
 }
@@ -958,7 +1060,8 @@ int se_gather(se_plan* p, const void* xyz, const void* q, void* phi, void* F, do
     if (!p || (p->N > 0 && (!xyz || !q))) return SE_ERR_ARG;
     if (!p->ready || !p->have_scale) return SE_ERR_ARG;
     if (p->variant >= 3) return fast_gather(p, phi, F, E);
-    return p->prec == SE_FP64 ? do_gather<double>(p, phi, F, E) : do_gather<float>(p, phi, F, E);
+    return p->prec == SE_FP64 ? do_gather<double>(p, xyz, q, phi, F, E)
+                              : do_gather<float>(p, xyz, q, phi, F, E);
 }
 
 int se_adjoint(se_plan* p, const void* xyz, const void* q, const double* gE, void* grad_x,
@@ -966,8 +1069,8 @@ int se_adjoint(se_plan* p, const void* xyz, const void* q, const double* gE, voi
     if (!p || !gE || (p->N > 0 && (!xyz || !q))) return SE_ERR_ARG;
     if (!p->ready || !p->have_scale) return SE_ERR_ARG;
     if (p->variant >= 3) return fast_gather(p, grad_q, grad_x, nullptr, gE);
-    return p->prec == SE_FP64 ? do_gather<double>(p, grad_q, grad_x, nullptr, gE)
-                              : do_gather<float>(p, grad_q, grad_x, nullptr, gE);
+    return p->prec == SE_FP64 ? do_gather<double>(p, xyz, q, grad_q, grad_x, nullptr, gE)
+                              : do_gather<float>(p, xyz, q, grad_q, grad_x, nullptr, gE);
 }
 
 int se_energy_force(se_plan* p, const void* xyz, const void* q, double* E, void* F, void* phi) {
