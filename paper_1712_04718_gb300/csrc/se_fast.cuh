@@ -251,6 +251,36 @@ __host__ __device__ constexpr int region_stride(int Rz) {
     return region_pad<P>() > 0 ? region_pad<P>() : Rz;
 }
 
+// Walk over the points of a staged region, nx planes of Ry x Rz points (origin
+// (ox, oy, oz) on the grid, rows RS apart, planes `plane` apart in the region), by
+// the whole block: body(w, g) with the point's index in the region and its
+// wrapped index in the grid.  A thread keeps its (y, z) and runs over the planes,
+// so that a point costs two additions instead of two divisions and three
+// wraps (about 20 instructions, which were half of the tile gather's: 639 ->
+// 372 us for the 64-box ensemble at P = 10, 38 -> 31 us for 100 200 atoms at
+// P = 8; the spread's flush 383 -> 349 and 34 -> 30 us).
+template <typename Body>
+__device__ __forceinline__ void region_walk(int nx, int Ry, int Rz, int RS, int plane, int ox,
+                                            int oy, int oz, int M, Body body) {
+    const FDiv fRz = fdiv_of(Rz);
+    const int M2 = M * M;
+    for (int e = threadIdx.x; e < Ry * Rz; e += blockDim.x) {
+        const int ry = fdiv(e, fRz), rz = e - ry * Rz;
+        int gx = wrap_index(ox, M);
+        int g = (gx * M + wrap_index(oy + ry, M)) * M + wrap_index(oz + rz, M);
+        int w = ry * RS + rz;
+#pragma unroll 4
+        for (int rx = 0; rx < nx; ++rx, w += plane) {
+            body(w, g);
+            g += M2;
+            if (++gx == M) {   // uniform
+                gx = 0;
+                g -= M2 * M;
+            }
+        }
+    }
+}
+
 // Spread of one tile (Eq. 3.5) into the fixed-point grid g64 (scale fxs =
 // 2^k): the n particles parts[0..n) of the tile.  The tile's region is
 // accumulated in shared memory as one 32-bit integer per point at the scale
@@ -358,20 +388,11 @@ __device__ __forceinline__ void spread_tile(const f4* __restrict__ parts, int n,
         }
         __syncthreads();
         SE_STAMP(2, 3);
-        const int ox = t0x - P / 2 + 1 + s0, oy = t0y - P / 2 + 1, oz = t0z - P / 2 + 1;
-        const FDiv fRz = fdiv_of(Rz), fRy = fdiv_of(Ry);
-        const int nlog = ns * Ry * Rz;   // the region's points, without the row padding
-        for (int e = threadIdx.x; e < nlog; e += blockDim.x) {
-            const int r = fdiv(e, fRz), rz = e - r * Rz;
-            const int w = (int)acc[r * RS + rz];
-            if (w != 0) {
-                const int rx = fdiv(r, fRy), ry = r - rx * Ry;
-                const int gx_ = wrap_index(ox + rx, M), gy_ = wrap_index(oy + ry, M),
-                          gz_ = wrap_index(oz + rz, M);
-                atomicAdd(g64 + ((size_t)gx_ * M + gy_) * M + gz_,
-                          (unsigned long long)((long long)w << shift));
-            }
-        }
+        region_walk(ns, Ry, Rz, RS, plane, t0x - P / 2 + 1 + s0, t0y - P / 2 + 1, t0z - P / 2 + 1,
+                    M, [&](int e, int g) {
+                        const int w = (int)acc[e];
+                        if (w != 0) atomicAdd(g64 + g, (unsigned long long)((long long)w << shift));
+                    });
         __syncthreads();
         SE_STAMP(2, 4);
     }
@@ -641,32 +662,15 @@ __device__ __forceinline__ void tile_accum(const TilePrep<P, DD>& g, const float
 
 // Copy the grid over a tile region (origin o = tile origin - P/2 + 1, extent
 // Rx x Ry x Rz, wrapped periodically) into shared memory, rows RS values
-// apart (RS >= Rz); the whole block.
+// apart (RS >= Rz), with asynchronous copies, all of a thread's in flight at
+// once; the whole block.
 __device__ __forceinline__ void load_region(const float* __restrict__ grid, int M, int ox, int oy,
                                             int oz, int Rx, int Ry, int Rz, int RS, float* reg) {
-    const int nel = Rx * Ry * Rz;
-    const FDiv fRz = fdiv_of(Rz), fRy = fdiv_of(Ry);
-    for (int e0 = threadIdx.x; e0 < nel; e0 += blockDim.x * kLoadBatch) {
-        float v[kLoadBatch];
-#pragma unroll
-        for (int u = 0; u < kLoadBatch; ++u) {
-            const int e = e0 + u * (int)blockDim.x;
-            if (e < nel) {
-                const int r = fdiv(e, fRz), rz = e - r * Rz;
-                const int rx = fdiv(r, fRy), ry = r - rx * Ry;
-                v[u] = __ldg(grid + ((size_t)wrap_index(ox + rx, M) * M + wrap_index(oy + ry, M)) * M +
-                             wrap_index(oz + rz, M));
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < kLoadBatch; ++u) {
-            const int e = e0 + u * (int)blockDim.x;
-            if (e < nel) {
-                const int r = fdiv(e, fRz);
-                reg[r * RS + (e - r * Rz)] = v[u];
-            }
-        }
-    }
+    region_walk(Rx, Ry, Rz, RS, Ry * RS, ox, oy, oz, M, [&](int e, int g) {
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(
+                         (unsigned)__cvta_generic_to_shared(reg + e)), "l"(grid + g) : "memory");
+    });
+    asm volatile("cp.async.wait_all;" ::: "memory");
 }
 
 // Sum over the G lanes of a particle, then lane 0 of the group writes phi and
