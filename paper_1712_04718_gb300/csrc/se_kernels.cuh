@@ -153,6 +153,32 @@ __device__ __forceinline__ double block_sum(double v, double* sbuf) {
     return r;  // valid in thread 0
 }
 
+// Block-wide sums of a and b (blockDim.x a multiple of 32, <= 512; sbuf: 32
+// values), valid in thread 0: half a warp carries each, so that a warp makes
+// five FP64 additions (each about 20 clocks of the SM's FP64 pipe) instead of
+// ten, and the warps' sums are added by a tree instead of one by one.
+__device__ __forceinline__ double2 block_sum2(double a, double b, double* sbuf) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const bool up = lane & 16;
+    double x = up ? b : a;
+    x += __shfl_xor_sync(0xffffffffu, up ? a : b, 16);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    __syncthreads();
+    if ((lane & 15) == 0) sbuf[(lane & 16) + warp] = x;
+    __syncthreads();
+    double2 r = make_double2(0.0, 0.0);
+    if (warp == 0) {
+        x = (lane & 15) < nw ? sbuf[lane] : 0.0;
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1)
+            if (o < nw) x += __shfl_xor_sync(0xffffffffu, x, o);
+        r.x = x;
+        r.y = __shfl_sync(0xffffffffu, x, 16);
+    }
+    return r;
+}
+
 // ---------------------------------------------------------------------------
 // Double-float sums: a value hi + lo held in two floats (about 48 significant
 // bits), added with two-sum.  The single-precision kernels reduce energies and
@@ -270,15 +296,18 @@ k_bin(const T* __restrict__ xyz, const T* __restrict__ q, const KParams<T> kp,
     __shared__ double sbuf[32];
     __shared__ unsigned long long sqm;
     __shared__ int s_tmax;
-    double sq = 0.0, sa = 0.0, bad = 0.0;
+    __shared__ int s_bad;
+    double sq = 0.0, sa = 0.0;
+    int bad = 0;
     unsigned long long qm = 0u;   // bits of the largest finite |q| (as a double)
     if (threadIdx.x == 0) {
         sqm = 0u;
         s_tmax = 0;
+        s_bad = 0;
     }
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < kp.N; i += gridDim.x * blockDim.x) {
         T x = xyz[3 * i], y = xyz[3 * i + 1], z = xyz[3 * i + 2], qq = q[i];
-        if (!(isfinite(x) && isfinite(y) && isfinite(z) && isfinite(qq))) bad += 1.0;
+        if (!(isfinite(x) && isfinite(y) && isfinite(z) && isfinite(qq))) ++bad;
         T t;
         int cx = cell_of(wrap_coord(x, kp.L, kp.invL), kp.invh, kp.M, &t);
         int cy = cell_of(wrap_coord(y, kp.L, kp.invL), kp.invh, kp.M, &t);
@@ -291,9 +320,8 @@ k_bin(const T* __restrict__ xyz, const T* __restrict__ q, const KParams<T> kp,
         const unsigned long long b = (unsigned long long)__double_as_longlong(fabs((double)qq));
         if (b < 0x7ff0000000000000ull && b > qm) qm = b;
     }
-    double r0 = block_sum(sq, sbuf);
-    double r1 = block_sum(sa, sbuf);
-    double r2 = block_sum(bad, sbuf);
+    const double2 r = block_sum2(sq, sa, sbuf);   // its barriers order the shared resets, too
+    if (bad) atomicAdd(&s_bad, bad);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         const unsigned long long v = __shfl_xor_sync(0xffffffffu, qm, o);
@@ -302,19 +330,28 @@ k_bin(const T* __restrict__ xyz, const T* __restrict__ q, const KParams<T> kp,
     if ((threadIdx.x & 31) == 0) atomicMax(&sqm, qm);
     __syncthreads();
     if (threadIdx.x == 0) {
-        partials[3 * blockIdx.x] = r0;
-        partials[3 * blockIdx.x + 1] = r1;
-        partials[3 * blockIdx.x + 2] = r2;
+        partials[3 * blockIdx.x] = r.x;
+        partials[3 * blockIdx.x + 1] = r.y;
+        partials[3 * blockIdx.x + 2] = __longlong_as_double(s_bad);
         qmax_part[blockIdx.x] = sqm;
     }
     if (!last_block(ticket)) return;
-    if (threadIdx.x == 0) sqm = 0u;
+    if (threadIdx.x == 0) {
+        sqm = 0u;
+        s_bad = 0;
+    }
     __syncthreads();
     qm = 0u;
+    sq = sa = 0.0;
+    bad = 0;
     for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) {
         const unsigned long long v = __ldcg(qmax_part + b);
         qm = v > qm ? v : qm;
+        sq += __ldcg(partials + 3 * b);
+        sa += __ldcg(partials + 3 * b + 1);
+        bad += (int)__double_as_longlong(__ldcg(partials + 3 * b + 2));
     }
+    if (bad) atomicAdd(&s_bad, bad);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         const unsigned long long v = __shfl_xor_sync(0xffffffffu, qm, o);
@@ -324,13 +361,11 @@ k_bin(const T* __restrict__ xyz, const T* __restrict__ q, const KParams<T> kp,
 
     // --- last block: checks, exclusive scan of the tile counts ---
     {
-        const double a = sum_partials(partials, gridDim.x, 3, 0, sbuf);
-        const double b = sum_partials(partials, gridDim.x, 3, 1, sbuf);
-        const double c = sum_partials(partials, gridDim.x, 3, 2, sbuf);
+        const double2 t = block_sum2(sq, sa, sbuf);
         if (threadIdx.x == 0) {
-            acc->sum_q = a;
-            acc->sum_absq = b;
-            acc->nonfinite = (unsigned)c;
+            acc->sum_q = t.x;
+            acc->sum_absq = t.y;
+            acc->nonfinite = (unsigned)s_bad;
             // the scale of the charges: |q| qscale < 1; charges below 2^-1000 keep 2^1000
             const double qmax = __longlong_as_double((long long)sqm);
             acc->qscale = qmax > 0x1p-1000 ? (1.0 - 0x1p-50) / qmax : 0x1p+1000;
