@@ -18,9 +18,8 @@ namespace {
 
 // The padded integer grid (units of 2^-grid_bits of the largest charge, times
 // c_g) -> FP64: every grid point is the sum of its images.  A warp takes a row
-// (x, y).  The integer grid is cleared by a memset afterwards: clearing what was
-// read here made the loads wait for the stores (113 us instead of 10 for 119^3
-// points).
+// (x, y).  The scaling step clears the integer grid: clearing what was read here
+// made the loads wait for the stores (113 us instead of 16 for 119^3 points).
 __global__ void __launch_bounds__(256)
 k_fx_fold(const long long* __restrict__ g, int Mp, int p0, const FxParams fp,
           const Acc* __restrict__ acc, double* __restrict__ grid) {
@@ -47,41 +46,26 @@ k_fx_fold(const long long* __restrict__ g, int Mp, int p0, const FxParams fp,
     }
 }
 
-// Largest high word (sign bit cleared) of the grid's values, per block.
-__global__ void __launch_bounds__(256)
-k_grid_top(const double* __restrict__ grid, long long n, unsigned* __restrict__ top) {
-    __shared__ unsigned m;
-    if (threadIdx.x == 0) m = 0u;
-    __syncthreads();
-    unsigned v = 0u;
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride)
-        v = max(v, (unsigned)__double2hiint(grid[i]) & 0x7fffffffu);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
-    if ((threadIdx.x & 31) == 0) atomicMax(&m, v);
-    __syncthreads();
-    if (threadIdx.x == 0) top[blockIdx.x] = m;
-}
-
 // The grid split in units of 2^(E - hb), every |value| < 2^E, by integer
 // operations on the bits, and padded by its periodic images to Mp^3 points,
 // Mp = M + P - 1, point (x, y, z) being grid point (x - p0, y - p0, z - p0) mod M.
-// Block 0 leaves the biased exponent E + 1022 in top[kFxTopBlocks].
+// E from the bound
+//   |Ht(x)| <= sum_k G/M^3 |Hhat| <= (sum_k G)^1/2 (sum_k G |Hhat|^2)^1/2 / M^3
+// (Cauchy and Schwarz; the second sum is the grid energy's, known from the
+// scaling step).  It exceeds the largest value by about sqrt(N) / 3, 6 bits of
+// the 60 at 21 642 atoms, and saves a pass over the grid.  Block 0 leaves the
+// biased exponent E + 1022 in *top.
 __global__ void __launch_bounds__(256)
-k_grid_split(const double* __restrict__ grid, int M, int Mp, int p0, unsigned* __restrict__ top,
-             int ntop, int hb, int2* __restrict__ out) {
-    __shared__ unsigned m;
-    if (threadIdx.x == 0) m = 0u;
+k_grid_split(const double* __restrict__ grid, int M, int Mp, int p0, double gbound,
+             const Acc* __restrict__ acc, int* __restrict__ top, int hb, int2* __restrict__ out) {
+    __shared__ int s_top;
+    if (threadIdx.x == 0) {
+        const double bound = gbound * sqrt(acc->e_grid);
+        s_top = min(0x7fe, max(1, (__double2hiint(bound) >> 20) & 0x7ff));
+        if (blockIdx.x == 0) *top = s_top;
+    }
     __syncthreads();
-    unsigned v = 0u;
-    for (int i = threadIdx.x; i < ntop; i += blockDim.x) v = max(v, top[i]);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
-    if ((threadIdx.x & 31) == 0) atomicMax(&m, v);
-    __syncthreads();
-    const int etop = max(1, (int)(m >> 20));   // biased exponent of the largest
-    if (blockIdx.x == 0 && threadIdx.x == 0) top[kFxTopBlocks] = (unsigned)etop;
+    const int etop = s_top;
     const int warps = gridDim.x * (blockDim.x >> 5), lane = threadIdx.x & 31;
     for (int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); r < Mp * Mp; r += warps) {
         const int x = r / Mp, y = r - x * Mp;
@@ -91,7 +75,7 @@ k_grid_split(const double* __restrict__ grid, int M, int Mp, int p0, unsigned* _
             const int e = (int)(b >> 52) & 0x7ff;
             const long long mant = (b & 0xfffffffffffffLL) | (e ? 1LL << 52 : 0LL);   // < 2^53
             // |value| = mant 2^(max(e,1) - 1075); hb + 32 bits below 2^E, E = etop - 1022
-            const int sh = etop - max(e, 1);
+            const int sh = max(0, etop - max(e, 1));
             long long f = hb + 32 >= 53 ? mant << (hb + 32 - 53) : mant >> (53 - hb - 32);
             f = sh < 63 ? f >> sh : 0;
             if (b < 0) f = -f;
@@ -134,10 +118,7 @@ cudaError_t fx_spread(const double* xyz, const double* q, const FxParams& fp, co
     if (e != cudaSuccess || only) return e;
     const int M = fp.kp.M;
     const int blocks = (int)std::min(((long long)M * M + 7) / 8, 8LL * 152);
-    const size_t Mp = (size_t)M + fp.kp.P - 1;
-    k_fx_fold<<<blocks, 256, 0, s>>>(b.g64, (int)Mp, fp.kp.P / 2 - 1, fp, b.acc, b.grid);
-    e = cudaMemsetAsync(b.g64, 0, Mp * Mp * Mp * sizeof(long long), s);
-    if (e != cudaSuccess) return e;
+    k_fx_fold<<<blocks, 256, 0, s>>>(b.g64, M + fp.kp.P - 1, fp.kp.P / 2 - 1, fp, b.acc, b.grid);
     return cudaGetLastError();
 }
 
@@ -145,13 +126,10 @@ cudaError_t fx_gather(const double* xyz, const double* q, const FxParams& fp, co
                       const double* grid, double* phi, double* F, double e_scale, double* E_out,
                       const double* adj, cudaStream_t s) {
     const int N = fp.kp.N;
-    const long long n = (long long)fp.kp.M * fp.kp.M * fp.kp.M;
-    const int ntop = (int)std::min((n + 1023) / 1024, (long long)kFxTopBlocks);
-    k_grid_top<<<ntop, 256, 0, s>>>(grid, n, b.top);
     const int Mp = fp.kp.M + fp.kp.P - 1;
     const int blocks = (int)std::min(((long long)Mp * Mp + 7) / 8, 8LL * 152);
-    k_grid_split<<<blocks, 256, 0, s>>>(grid, fp.kp.M, Mp, fp.kp.P / 2 - 1, b.top, ntop, fp.hb,
-                                        (int2*)b.split);
+    k_grid_split<<<blocks, 256, 0, s>>>(grid, fp.kp.M, Mp, fp.kp.P / 2 - 1, fp.gbound, b.acc,
+                                        b.top, fp.hb, (int2*)b.split);
     cudaError_t e = cudaGetLastError();
     for (int c0 = 0; e == cudaSuccess; c0 += b.cap) {
         const int c1 = (int)std::min<long long>(N, (long long)c0 + b.cap);

@@ -17,8 +17,7 @@
 //                   that no support wraps, with global reductions: integer
 //                   sums, the same for every order
 //   k_fx_fold       integer grid -> FP64, its periodic images added
-//   k_grid_top, k_grid_split   largest exponent of the transformed grid, and
-//                   the grid split at that scale, padded by its periodic images
+//   k_grid_split    the transformed grid split, padded by its periodic images
 //   k_gather_fx     Eq. 3.9 and the forces: y, x and z sums as above, one
 //                   conversion to FP64 per particle and result
 //
@@ -246,7 +245,7 @@ template <int P>
 __global__ void __launch_bounds__(P <= 16 ? 256 : 512, P == 14 || P == 16 ? 1 : 2)
 k_gather_fx(const int4* __restrict__ fac, const int* __restrict__ cells,
             const double* __restrict__ sorted, const int* __restrict__ perm,
-            const int2* __restrict__ grid, const unsigned* __restrict__ top,
+            const int2* __restrict__ grid, const int* __restrict__ top,
             double* __restrict__ phi, double* __restrict__ F, const FxParams fp,
             double* __restrict__ parts, unsigned* ticket, Acc* acc, double e_scale, double* E_out,
             const double* __restrict__ adj, int c0, int c1) {
@@ -259,7 +258,7 @@ k_gather_fx(const int4* __restrict__ fac, const int* __restrict__ cells,
     const int Mp = kp.M + P - 1;
     // the grid's units 2^(E - hb); the sums are scaled by 2^30 per window and
     // cut by 2^(32 + e1) and 2^(32 + e2)
-    const double unit = pow2i((int)top[0] - 1022 - fp.hb - 26 + fp.e1 + fp.e2);
+    const double unit = pow2i(top[0] - 1022 - fp.hb - 26 + fp.e1 + fp.e2);
     const double gsc = adj ? __ldg(adj) : 1.0;
     const double u_phi = unit * kp.phi_scale;
     const double u_F = unit * kp.F_scale * pow2i(fp.sd) * (adj ? -gsc : 1.0);

@@ -34,7 +34,7 @@ cudaError_t fx_gather_P(const FxParams& fp, const FxBufs& b, double* phi, double
     const int blocks = std::max(1, std::min((warps_all + warps - 1) / warps, b.nparts));
     k_gather_fx<P><<<blocks, 32 * warps, 0, s>>>(
         (const int4*)b.fac, b.cells, (const double*)b.sorted, b.perm, (const int2*)b.split,
-        b.top + kFxTopBlocks, phi, F, fp, b.parts, b.ticket, b.acc, e_scale, E_out, adj, c0, c1);
+        b.top, phi, F, fp, b.parts, b.ticket, b.acc, e_scale, E_out, adj, c0, c1);
     return cudaGetLastError();
 }
 

@@ -65,7 +65,7 @@ template <typename T>
 cudaError_t launch_spread_direct(const v4_t<T>* sorted, T* grid, const KParams<T>& kp,
                                  cudaStream_t s);
 template <typename T>
-cudaError_t launch_scale(void* cgrid, const double* green, int M, T* zero_grid,
+cudaError_t launch_scale(void* cgrid, const double* green, int M, T* zero_grid, long long nzero,
                          double* partials, unsigned* ticket, Acc* acc, double e_scale,
                          double* E_out, cudaStream_t s);
 template <typename T>
@@ -79,8 +79,8 @@ cudaError_t launch_gather(const v4_t<T>* sorted, const int* perm, const T* grid,
 // complex half spectrum, dstride >= M^2 (M/2+1) complex values apart).
 template <typename T>
 cudaError_t launch_scale_ik(void* cgrid, void* dgrid, size_t dstride, const double* green, int M,
-                            double L, T* zero_grid, double* partials, unsigned* ticket, Acc* acc,
-                            double e_scale, double* E_out, cudaStream_t s);
+                            double L, T* zero_grid, long long nzero, double* partials, unsigned* ticket,
+                            Acc* acc, double e_scale, double* E_out, cudaStream_t s);
 // Gather with the underived window from ng grids gstride values apart:
 // ng = 1 potential (and energy) only; ng = 4 potential and ik forces from
 // [Ht, dHt/dx, dHt/dy, dHt/dz].  pdl: launched as a programmatic dependent.
@@ -97,10 +97,10 @@ struct FxParams {
     int sd;           // 2^sd bounds the derivative window's factors
     int hb;           // integer bits of the split grid
     float crowd;      // see grid_bits
+    double gbound;    // sqrt(sum_k G) / M^3: times sqrt(sum_k G |H^|^2), a bound of the grid
     int e1, e2;       // the gather's sums over y and x are cut by 32 + e1, 32 + e2 bits
 };
 constexpr size_t kFxFactorBytes = (size_t)4 << 30;   // window factors of one range of particles
-constexpr int kFxTopBlocks = 512;
 struct FxBufs {
     long long* g64;        // (M + P - 1)^3: the integer grid, zero between calls
     double* grid;          // M^3: the FP64 spread grid
@@ -111,7 +111,7 @@ struct FxBufs {
     int *slot, *tile_of, *tile_start, *perm;
     void* sorted;          // d4 [N]
     void* split;           // int2 [(M + P - 1)^3]: the transformed grid, split and padded
-    unsigned* top;         // [kFxTopBlocks]: per-block largest high words, then the exponent
+    int* top;              // biased exponent of the split grid's bound
     double* parts;         // [nparts] energy partials
     int nparts;
     unsigned* ticket;

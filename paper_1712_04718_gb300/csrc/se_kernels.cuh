@@ -628,14 +628,14 @@ k_spread_direct(const v4_t<T>* __restrict__ sorted, T* __restrict__ grid, const 
 // ---------------------------------------------------------------------------
 // a5: scale.  Hhat <- G(k)/M^3 Hhat on the half spectrum, the grid energy
 // sum_k w_k G |Hhat|^2 (w = 1 on the kz = 0 and Nyquist planes, 2 elsewhere),
-// and zeroing of the spread grid for the next spread (the forward FFT has
-// consumed it).  G is an FP64 table.
+// and zeroing of the nzero values of the spread grid for the next spread (it has
+// been consumed).  G is an FP64 table.
 // ---------------------------------------------------------------------------
 template <typename T, typename C>
 __global__ void __launch_bounds__(256)
 k_scale(C* __restrict__ cgrid, const double* __restrict__ green, int M, double invM3,
-        T* __restrict__ zero_grid, double* __restrict__ partials, unsigned* ticket,
-        Acc* acc, double e_scale, double* E_out) {
+        T* __restrict__ zero_grid, long long nzero, double* __restrict__ partials,
+        unsigned* ticket, Acc* acc, double e_scale, double* E_out) {
     __shared__ double sbuf[32];
     const int Mh = M / 2 + 1;
     const long long total = (long long)M * M * Mh;
@@ -653,8 +653,7 @@ k_scale(C* __restrict__ cgrid, const double* __restrict__ green, int M, double i
         cgrid[i] = c;
     }
     if (zero_grid) {
-        const long long n3 = (long long)M * M * M;
-        for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n3; i += stride)
+        for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < nzero; i += stride)
             zero_grid[i] = T(0);
     }
     double r = block_sum(e, sbuf);

@@ -88,7 +88,7 @@ cudaError_t launch_spread_direct(const v4_t<T>* sorted, T* grid, const KParams<T
 }
 
 template <typename T>
-cudaError_t launch_scale(void* cgrid, const double* green, int M, T* zero_grid,
+cudaError_t launch_scale(void* cgrid, const double* green, int M, T* zero_grid, long long nzero,
                          double* partials, unsigned* ticket, Acc* acc, double e_scale,
                          double* E_out, cudaStream_t s) {
     using C = typename std::conditional<std::is_same<T, float>::value, float2, double2>::type;
@@ -96,7 +96,7 @@ cudaError_t launch_scale(void* cgrid, const double* green, int M, T* zero_grid,
     const int blocks = (int)std::max(1LL, std::min((total + kThreads - 1) / kThreads,
                                                    (long long)kMaxPartials));
     const double invM3 = 1.0 / ((double)M * M * M);
-    k_scale<T, C><<<blocks, kThreads, 0, s>>>((C*)cgrid, green, M, invM3, zero_grid, partials,
+    k_scale<T, C><<<blocks, kThreads, 0, s>>>((C*)cgrid, green, M, invM3, zero_grid, nzero, partials,
                                               ticket, acc, e_scale, E_out);
     return cudaGetLastError();
 }
@@ -136,8 +136,8 @@ cudaError_t launch_gather(const v4_t<T>* sorted, const int* perm, const T* grid,
                                                 const KParams<T>&, bool, cudaStream_t);         \
     template cudaError_t launch_spread_direct<T>(const v4_t<T>*, T*, const KParams<T>&,         \
                                                  cudaStream_t);                                 \
-    template cudaError_t launch_scale<T>(void*, const double*, int, T*, double*, unsigned*,     \
-                                         Acc*, double, double*, cudaStream_t);
+    template cudaError_t launch_scale<T>(void*, const double*, int, T*, long long, double*,     \
+                                         unsigned*, Acc*, double, double*, cudaStream_t);
 #define SE_INSTANTIATE_GATHER(T)                                                                \
     template cudaError_t launch_gather<T>(const v4_t<T>*, const int*, const T*, T*, T*,         \
                                           const KParams<T>&, double*, unsigned*, Acc*, double,  \

@@ -37,8 +37,8 @@ template <typename T, typename C>
 __global__ void __launch_bounds__(256)
 k_scale_ik(C* __restrict__ cgrid, C* __restrict__ dgrid, long long dstride,
            const double* __restrict__ green, int M, double invM3, double kunit,
-           T* __restrict__ zero_grid, double* __restrict__ partials, unsigned* ticket, Acc* acc,
-           double e_scale, double* E_out) {
+           T* __restrict__ zero_grid, long long nzero, double* __restrict__ partials,
+           unsigned* ticket, Acc* acc, double e_scale, double* E_out) {
     __shared__ double sbuf[32];
     const int Mh = M / 2 + 1;
     const long long total = (long long)M * M * Mh;
@@ -73,8 +73,7 @@ k_scale_ik(C* __restrict__ cgrid, C* __restrict__ dgrid, long long dstride,
         cgrid[i] = c;
     }
     if (zero_grid) {
-        const long long n3 = (long long)M * M * M;
-        for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n3; i += stride)
+        for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < nzero; i += stride)
             zero_grid[i] = T(0);
     }
     double rs = block_sum(e, sbuf);
@@ -232,8 +231,8 @@ k_gather_plain(const v4_t<T>* __restrict__ sorted, const int* __restrict__ perm,
 
 template <typename T>
 cudaError_t launch_scale_ik(void* cgrid, void* dgrid, size_t dstride, const double* green, int M,
-                            double L, T* zero_grid, double* partials, unsigned* ticket, Acc* acc,
-                            double e_scale, double* E_out, cudaStream_t s) {
+                            double L, T* zero_grid, long long nzero, double* partials, unsigned* ticket,
+                            Acc* acc, double e_scale, double* E_out, cudaStream_t s) {
     using C = typename std::conditional<std::is_same<T, float>::value, float2, double2>::type;
     const long long total = (long long)M * M * (M / 2 + 1);
     const int blocks = (int)std::max(1LL, std::min((total + 255) / 256, (long long)kMaxPartials));
@@ -241,7 +240,7 @@ cudaError_t launch_scale_ik(void* cgrid, void* dgrid, size_t dstride, const doub
     const double kunit = 2.0 * 3.14159265358979323846 / L;
     if (dstride < (size_t)total) return cudaErrorInvalidValue;
     k_scale_ik<T, C><<<blocks, 256, 0, s>>>((C*)cgrid, (C*)dgrid, (long long)dstride, green, M,
-                                             invM3, kunit, zero_grid, partials, ticket, acc,
+                                             invM3, kunit, zero_grid, nzero, partials, ticket, acc,
                                              e_scale, E_out);
     return cudaGetLastError();
 }
@@ -287,8 +286,8 @@ cudaError_t launch_gather_plain(int ng, const v4_t<T>* sorted, const int* perm, 
 
 #define SE_PLAIN_INSTANTIATE(T)                                                                 \
     template cudaError_t launch_scale_ik<T>(void*, void*, size_t, const double*, int, double,   \
-                                            T*, double*, unsigned*, Acc*, double, double*,      \
-                                            cudaStream_t);                                      \
+                                            T*, long long, double*, unsigned*, Acc*, double,    \
+                                            double*, cudaStream_t);                             \
     template cudaError_t launch_gather_plain<T>(int, const v4_t<T>*, const int*, const T*,      \
                                                 size_t, T*, T*, const KParams<T>&, double*,     \
                                                 unsigned*, Acc*, double, double*, bool,         \

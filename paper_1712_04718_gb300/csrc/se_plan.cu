@@ -86,7 +86,10 @@ struct se_plan {
     void* fx_xq = nullptr;
     int fx_cap = 0;
     int* fx_cells = nullptr;
-    unsigned* fx_top = nullptr;
+    int* fx_top = nullptr;
+    double fx_gbound = 0.0;
+    cudaStream_t fft_stream = nullptr;   // stream the FFT plans were last given
+    bool fft_stream_set = false;
     void* fx_split = nullptr;
     void* fx_grid = nullptr;
     double* fx_parts = nullptr;
@@ -241,6 +244,7 @@ void release_device(se_plan* p) {
         cufftDestroy(p->fwd);
         cufftDestroy(p->inv);
         p->have_fft = false;
+        p->fft_stream_set = false;
     }
     void* bufs[] = {p->grid_spread, p->grid_gather, p->cgrid, p->green, p->tile_count,
                     p->tile_start, p->slot, p->tile_of, p->perm, p->sorted, p->partials,
@@ -372,7 +376,7 @@ int prepare(se_plan* p) {
         if (rc == SE_OK) rc = dalloc(&p->fx_fac, (size_t)p->fx_cap * 48 * p->P);
         if (rc == SE_OK) rc = dalloc(&p->fx_xq, (size_t)p->fx_cap * 8 * p->P);
         if (rc == SE_OK) rc = dalloc((void**)&p->fx_cells, N * 4 * sizeof(int));
-        if (rc == SE_OK) rc = dalloc((void**)&p->fx_top, (se::kFxTopBlocks + 1) * sizeof(unsigned));
+        if (rc == SE_OK) rc = dalloc((void**)&p->fx_top, sizeof(int));
         const size_t Mp = (size_t)p->M + p->P - 1;
         if (rc == SE_OK) rc = dalloc(&p->fx_split, Mp * Mp * Mp * 2 * sizeof(int));
         if (rc == SE_OK) rc = dalloc(&p->fx_grid, Mp * Mp * Mp * sizeof(long long));
@@ -386,6 +390,14 @@ int prepare(se_plan* p) {
         return rc;
     }
     std::vector<double> g = green_table(p);
+    if (p->prec == SE_FP64) {
+        // sum of G over the whole spectrum: the half spectrum's inner planes twice
+        double sum = 0.0;
+        const int Mh = p->M / 2 + 1;
+        for (size_t i = 0; i < nc; i += Mh)
+            for (int k = 0; k < Mh; ++k) sum += (k == 0 || 2 * k == p->M ? 1.0 : 2.0) * g[i + k];
+        p->fx_gbound = sqrt(sum) / (double)M3 * (1.0 + 1e-6);
+    }
     if (cudaMemcpy(p->green, g.data(), nc * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess ||
         cudaMemset(p->tile_count, 0, (size_t)p->ntiles * sizeof(int)) != cudaSuccess ||
         cudaMemset(p->tickets, 0, 8 * sizeof(unsigned)) != cudaSuccess ||
@@ -450,6 +462,22 @@ void invalidate(se_plan* p) {
     derive(p);
 }
 
+// The grid that the spread adds to: the fixed-point one of the single-precision
+// pipeline, the padded integer one of the double-precision spread, or the real
+// one; and its values (all of 8 bytes but for float grids).
+bool fx_spread_used(const se_plan* p) { return p->prec == SE_FP64 && p->variant != 2; }
+void* spread_target(const se_plan* p, size_t* n) {
+    const size_t e = (size_t)p->M + (fx_spread_used(p) ? p->P - 1 : 0);
+    *n = e * e * e;
+    return p->variant >= 3 ? (void*)p->g64 : (fx_spread_used(p) ? p->fx_grid : p->grid_spread);
+}
+int clear_spread(se_plan* p) {
+    size_t n = 0;
+    void* g = spread_target(p, &n);
+    const size_t each = p->variant >= 3 ? sizeof(long long) : tsize(p->prec);
+    return check_cuda(cudaMemsetAsync(g, 0, n * each, p->stream));
+}
+
 se::FastBufs fast_bufs(se_plan* p) {
     se::FastBufs b;
     b.g64 = p->g64;
@@ -494,6 +522,7 @@ se::FxParams fx_params(const se_plan* p) {
     double k = 0.0;
     for (int i = 0; i * p->tile <= p->P; ++i) k += 2.0 * exp(-beta * i * p->tile * i * p->tile);
     f.crowd = (float)(k * k * k * (1.0 + 1e-6));
+    f.gbound = p->fx_gbound;
     f.hb = std::min(30, (int)floor(top - 30.0 - gs));
     const double s1 = 30.0 + f.hb + gs;                              // sum over y
     f.e1 = std::max(0, (int)ceil(30.0 + gs + s1 - 32.0 - top));
@@ -531,8 +560,7 @@ int fast_spread(se_plan* p, const void* xyz, const void* q) {
     const KParams<float> kp = make_kparams<float>(p);
     // the spread adds into g64 (fixed point, or float with variant 4), which
     // the forward slab kernel clears as it reads it
-    if (!p->spread_clean)
-        SE_CUDA(cudaMemsetAsync(p->g64, 0, (size_t)p->M * p->M * p->M * sizeof(long long), p->stream));
+    if (!p->spread_clean) SE_TRY(clear_spread(p));
     p->spread_clean = false;
     timing_begin(p);
     SE_CUDA(se::fast_spread((const float*)xyz, (const float*)q, kp, fast_bufs(p), p->stream,
@@ -596,11 +624,7 @@ template <typename T>
 int do_spread(se_plan* p, const void* xyz, const void* q) {
     const KParams<T> kp = make_kparams<T>(p);
     using V = se::v4_t<T>;
-    const size_t M3 = (size_t)p->M * p->M * p->M;
-    // the integer spread overwrites the FP64 grid; the others add to it
-    const bool adds = std::is_same<T, float>::value || p->variant == 2;
-    if (adds && !p->spread_clean)
-        SE_CUDA(cudaMemsetAsync(p->grid_spread, 0, M3 * sizeof(T), p->stream));
+    if (!p->spread_clean) SE_TRY(clear_spread(p));
     timing_begin(p);
     SE_CUDA(se::launch_bin<T>((const T*)xyz, (const T*)q, kp, p->tile_count, p->slot, p->tile_of,
                               p->tile_start, p->partials, p->tickets + 0, p->acc, p->stream));
@@ -633,8 +657,12 @@ int do_spread(se_plan* p, const void* xyz, const void* q) {
 
 template <typename T>
 int do_scale(se_plan* p, double* E_grid) {
-    SE_CUFFT(cufftSetStream(p->fwd, p->stream));
-    SE_CUFFT(cufftSetStream(p->inv, p->stream));
+    if (!p->fft_stream_set || p->fft_stream != p->stream) {
+        SE_CUFFT(cufftSetStream(p->fwd, p->stream));
+        SE_CUFFT(cufftSetStream(p->inv, p->stream));
+        p->fft_stream = p->stream;
+        p->fft_stream_set = true;
+    }
     if (p->prec == SE_FP64)
         SE_CUFFT(cufftExecD2Z(p->fwd, (cufftDoubleReal*)p->grid_spread, (cufftDoubleComplex*)p->cgrid));
     else
@@ -643,15 +671,15 @@ int do_scale(se_plan* p, double* E_grid) {
     const double M3 = (double)p->M * p->M * p->M;
     const double e_scale = p->kc * p->h * p->h * p->h / (2.0 * M3);
     const bool ik = p->force_mode == SE_FORCE_IK;
-    // cleared for the next spread, unless that overwrites it
-    T* zero = std::is_same<T, float>::value || p->variant == 2 ? (T*)p->grid_spread : nullptr;
+    size_t nzero = 0;
+    T* zero = (T*)spread_target(p, &nzero);   // cleared for the next spread
     if (ik)
         SE_CUDA(se::launch_scale_ik<T>(p->cgrid, p->cgrid_ik, ik_cstride(p), p->green, p->M, p->L,
-                                       zero,
+                                       zero, (long long)nzero,
                                        p->partials + 3 * se::kMaxPartials, p->tickets + 1, p->acc,
                                        e_scale, E_grid, p->stream));
     else
-        SE_CUDA(se::launch_scale<T>(p->cgrid, p->green, p->M, zero, p->partials + 3 * se::kMaxPartials,
+        SE_CUDA(se::launch_scale<T>(p->cgrid, p->green, p->M, zero, (long long)nzero, p->partials + 3 * se::kMaxPartials,
                                     p->tickets + 1, p->acc, e_scale, E_grid, p->stream));
     timing_mark(p, 4);
     p->spread_clean = true;
@@ -744,18 +772,14 @@ int graph_evaluate(se_plan* p, const void* xyz, const void* q, void* F, void* ph
     const void* key[5] = {xyz, q, F, phi, dE};
     bool match = p->gexec && p->gkey_kc == p->kc;
     for (int i = 0; i < 5 && match; ++i) match = key[i] == p->gkey[i];
+    if (!p->spread_clean) {   // a spread that no scaling step followed
+        SE_TRY(clear_spread(p));
+        p->spread_clean = true;
+    }
     if (!match) {
         drop_graph(p);
         if (!p->cap_stream)
             SE_CUDA(cudaStreamCreateWithFlags(&p->cap_stream, cudaStreamNonBlocking));
-        if (!p->spread_clean) {
-            const size_t M3 = (size_t)p->M * p->M * p->M;
-            if (p->variant >= 3)
-                SE_CUDA(cudaMemsetAsync(p->g64, 0, M3 * sizeof(long long), p->stream));
-            else
-                SE_CUDA(cudaMemsetAsync(p->grid_spread, 0, M3 * tsize(p->prec), p->stream));
-            p->spread_clean = true;
-        }
         // the capture stream must see the state the user stream has reached
         SE_CUDA(cudaStreamSynchronize(p->stream));
         cudaStream_t user = p->stream;
@@ -823,6 +847,10 @@ int graph_evaluate_host(se_plan* p, const void* xyz, const void* q, void* F, voi
     const void* key[4] = {xyz, q, F, phi};
     bool match = p->hexec && p->hkey_kc == p->kc;
     for (int i = 0; i < 4 && match; ++i) match = key[i] == p->hkey[i];
+    if (!p->spread_clean) {   // a spread that no scaling step followed
+        SE_TRY(clear_spread(p));
+        p->spread_clean = true;
+    }
     if (!match) {
         if (p->hexec) cudaGraphExecDestroy(p->hexec);
         p->hexec = nullptr;
@@ -839,14 +867,6 @@ int graph_evaluate_host(se_plan* p, const void* xyz, const void* q, void* F, voi
         }
         if (!p->cap_stream)
             SE_CUDA(cudaStreamCreateWithFlags(&p->cap_stream, cudaStreamNonBlocking));
-        if (!p->spread_clean) {
-            const size_t M3 = (size_t)p->M * p->M * p->M;
-            if (p->variant >= 3)
-                SE_CUDA(cudaMemsetAsync(p->g64, 0, M3 * sizeof(long long), p->stream));
-            else
-                SE_CUDA(cudaMemsetAsync(p->grid_spread, 0, M3 * tsize(p->prec), p->stream));
-            p->spread_clean = true;
-        }
         SE_CUDA(cudaStreamSynchronize(p->stream));
         cudaStream_t user = p->stream;
         p->stream = p->cap_stream;
