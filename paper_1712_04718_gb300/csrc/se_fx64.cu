@@ -1,5 +1,7 @@
 // se_fx64.cu -- the double-precision integer spread and gather (se_fx64.cuh):
 // dispatch over the support and over ranges of particles.
+#include <math_constants.h>
+
 #include "se_fx64_launch.cuh"
 
 namespace se {
@@ -23,7 +25,9 @@ namespace {
 __global__ void __launch_bounds__(256)
 k_fx_fold(const long long* __restrict__ g, int Mp, int p0, const FxParams fp,
           const Acc* __restrict__ acc, double* __restrict__ grid) {
-    const double unit = fp.kp.qcg * acc->qunit * pow2i(-grid_bits(acc, fp));
+    // NaN or infinite input: NaN results, as the FP64 arithmetic gave
+    const double unit = acc->nonfinite ? CUDART_NAN
+                                       : fp.kp.qcg * acc->qunit * pow2i(-grid_bits(acc, fp));
     const int M = fp.kp.M, warps = gridDim.x * (blockDim.x >> 5), lane = threadIdx.x & 31;
     // the images of index i: i + p0, and one more M above or below (P <= M)
     auto other = [&](int i) { return i <= p0 ? i + p0 + M : (i >= M - p0 ? i + p0 - M : -1); };
@@ -53,14 +57,18 @@ k_fx_fold(const long long* __restrict__ g, int Mp, int p0, const FxParams fp,
 //   |Ht(x)| <= sum_k G/M^3 |Hhat| <= (sum_k G)^1/2 (sum_k G |Hhat|^2)^1/2 / M^3
 // (Cauchy and Schwarz; the second sum is the grid energy's, known from the
 // scaling step).  It exceeds the largest value by about sqrt(N) / 3, 6 bits of
-// the 60 at 21 642 atoms, and saves a pass over the grid.  Block 0 leaves the
-// biased exponent E + 1022 in *top.
+// the 60 at 21 642 atoms, and saves a pass over the grid.  Charges so large or
+// small that the energy leaves the normal range (beyond about 1e+-145) take
+//   |Ht(x)| <= sum_k G/M^3 sum_x |H(x)|,  sum_x |H| <= sum_n |q_n| c_g W^3
+// instead, W a bound of the sum of a window's factors (gbound1).  Block 0 leaves
+// the biased exponent E + 1022 in *top.
 __global__ void __launch_bounds__(256)
 k_grid_split(const double* __restrict__ grid, int M, int Mp, int p0, double gbound,
-             const Acc* __restrict__ acc, int* __restrict__ top, int hb, int2* __restrict__ out) {
+             double gbound1, const Acc* __restrict__ acc, int* __restrict__ top, int hb, int2* __restrict__ out) {
     __shared__ int s_top;
     if (threadIdx.x == 0) {
-        const double bound = gbound * sqrt(acc->e_grid);
+        const double e = acc->e_grid;
+        const double bound = e > 1e-290 && e < 1e300 ? gbound * sqrt(e) : gbound1 * acc->sum_absq;
         s_top = min(0x7fe, max(1, (__double2hiint(bound) >> 20) & 0x7ff));
         if (blockIdx.x == 0) *top = s_top;
     }
@@ -128,8 +136,8 @@ cudaError_t fx_gather(const double* xyz, const double* q, const FxParams& fp, co
     const int N = fp.kp.N;
     const int Mp = fp.kp.M + fp.kp.P - 1;
     const int blocks = (int)std::min(((long long)Mp * Mp + 7) / 8, 8LL * 152);
-    k_grid_split<<<blocks, 256, 0, s>>>(grid, fp.kp.M, Mp, fp.kp.P / 2 - 1, fp.gbound, b.acc,
-                                        b.top, fp.hb, (int2*)b.split);
+    k_grid_split<<<blocks, 256, 0, s>>>(grid, fp.kp.M, Mp, fp.kp.P / 2 - 1, fp.gbound,
+                                        fp.gbound1, b.acc, b.top, fp.hb, (int2*)b.split);
     cudaError_t e = cudaGetLastError();
     for (int c0 = 0; e == cudaSuccess; c0 += b.cap) {
         const int c1 = (int)std::min<long long>(N, (long long)c0 + b.cap);

@@ -32,6 +32,8 @@
 // Particles are taken in ranges of the tile order, so that the factors
 // (56 P bytes a particle) never need more than kFxFactorBytes.
 #pragma once
+#include <math_constants.h>
+
 #include <algorithm>
 
 #include "se_kernels.cuh"
@@ -257,8 +259,10 @@ k_gather_fx(const int4* __restrict__ fac, const int* __restrict__ cells,
     const int gi = lane / P, k = lane - gi * P;
     const int Mp = kp.M + P - 1;
     // the grid's units 2^(E - hb); the sums are scaled by 2^30 per window and
-    // cut by 2^(32 + e1) and 2^(32 + e2)
-    const double unit = pow2i(top[0] - 1022 - fp.hb - 26 + fp.e1 + fp.e2);
+    // cut by 2^(32 + e1) and 2^(32 + e2); NaN where an input was NaN or infinite
+    const double unit = acc->nonfinite
+                            ? CUDART_NAN
+                            : pow2i(top[0] - 1022 - fp.hb - 26 + fp.e1 + fp.e2);
     const double gsc = adj ? __ldg(adj) : 1.0;
     const double u_phi = unit * kp.phi_scale;
     const double u_F = unit * kp.F_scale * pow2i(fp.sd) * (adj ? -gsc : 1.0);

@@ -98,6 +98,7 @@ struct FxParams {
     int hb;           // integer bits of the split grid
     float crowd;      // see grid_bits
     double gbound;    // sqrt(sum_k G) / M^3: times sqrt(sum_k G |H^|^2), a bound of the grid
+    double gbound1;   // times sum |q|, another one
     int e1, e2;       // the gather's sums over y and x are cut by 32 + e1, 32 + e2 bits
 };
 constexpr size_t kFxFactorBytes = (size_t)4 << 30;   // window factors of one range of particles

@@ -523,6 +523,8 @@ se::FxParams fx_params(const se_plan* p) {
     for (int i = 0; i * p->tile <= p->P; ++i) k += 2.0 * exp(-beta * i * p->tile * i * p->tile);
     f.crowd = (float)(k * k * k * (1.0 + 1e-6));
     f.gbound = p->fx_gbound;
+    const double M3 = (double)p->M * p->M * p->M;   // fx_gbound^2 M^3 = sum_k G / M^3
+    f.gbound1 = p->fx_gbound * p->fx_gbound * M3 * f.kp.qcg * g * g * g;
     f.hb = std::min(30, (int)floor(top - 30.0 - gs));
     const double s1 = 30.0 + f.hb + gs;                              // sum over y
     f.e1 = std::max(0, (int)ceil(30.0 + gs + s1 - 32.0 - top));

@@ -2,7 +2,8 @@
 numbers) where they can go wrong: every support, tile edges with constant and
 with run-time row strides, several x-slabs a tile, more particles a tile than
 one round of the integer words takes, few particles, charges far from one,
-flat windows (the gather's scales), and several ranges of particles.
+flat windows (the gather's scales), several ranges of particles, and input
+beyond the range or not finite.
 
 Tolerances as the other FP64 comparisons: 1e-12 for the grid (weights are
 multiples of 2^-52 of the largest charge's), 5e-12 for particle outputs."""
@@ -129,3 +130,42 @@ def test_several_ranges():
     assert abs(E - Eg.item()) < 5 * TOL * abs(E)
     whole.close()
     part.close()
+
+
+@pytest.mark.parametrize("scale", [1e-200, 1e-150, 1e150, 1e200])
+def test_potential_beyond_the_energys_range(scale):
+    """Charges whose energy underflows or overflows still have a potential."""
+    L, xi, M, P = 2.0, 3.0, 24, 8
+    x, q = systems.uniform_charges(200, L, seed=5)
+    plan = se.Plan(len(q), L, xi, M, P, precision="fp64")
+    xd, qd = torch.tensor(x, device="cuda"), torch.tensor(q * scale, device="cuda")
+    F, phi = torch.empty_like(xd), torch.empty_like(qd)
+    plan.evaluate(xd, qd, F, phi)
+    torch.cuda.synchronize()
+    plan.close()
+    r = oracle.se_kspace(x, q, L, xi, M, P, cell_mode=64)
+    assert_close(phi.cpu().numpy() / scale, r["phi"], 5 * TOL, label="phi")
+
+
+@pytest.mark.parametrize("where,value", [("x", float("nan")), ("x", float("inf")),
+                                         ("q", float("nan")), ("q", float("-inf"))])
+def test_nonfinite_input_gives_nan(where, value):
+    """A call that does not read the status sees it in the results, and the
+    next call with finite input is as any other."""
+    L, xi, M, P = 2.0, 3.0, 24, 8
+    x, q = systems.uniform_charges(200, L, seed=5)
+    plan = se.Plan(len(q), L, xi, M, P, precision="fp64")
+    xd, qd = torch.tensor(x, device="cuda"), torch.tensor(q, device="cuda")
+    F, phi = torch.empty_like(xd), torch.empty_like(qd)
+    E = torch.zeros(1, dtype=torch.float64, device="cuda")
+    xb, qb = xd.clone(), qd.clone()
+    if where == "x":
+        xb[7, 1] = value
+    else:
+        qb[7] = value
+    plan.evaluate(xb, qb, F, phi, E)
+    assert bool(F.isnan().all()) and bool(phi.isnan().all()) and bool(E.isnan())
+    plan.evaluate(xd, qd, F, phi, E)
+    r = oracle.se_kspace(x, q, L, xi, M, P, cell_mode=64)
+    assert_close(phi.cpu().numpy(), r["phi"], 5 * TOL, label="phi")
+    plan.close()
