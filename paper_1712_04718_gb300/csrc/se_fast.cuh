@@ -251,36 +251,6 @@ __host__ __device__ constexpr int region_stride(int Rz) {
     return region_pad<P>() > 0 ? region_pad<P>() : Rz;
 }
 
-// Walk over the points of a staged region, nx planes of Ry x Rz points (origin
-// (ox, oy, oz) on the grid, rows RS apart, planes `plane` apart in the region), by
-// the whole block: body(w, g) with the point's index in the region and its
-// wrapped index in the grid.  A thread keeps its (y, z) and runs over the planes,
-// so that a point costs two additions instead of two divisions and three
-// wraps (about 20 instructions, which were half of the tile gather's: 639 ->
-// 372 us for the 64-box ensemble at P = 10, 38 -> 31 us for 100 200 atoms at
-// P = 8; the spread's flush 383 -> 349 and 34 -> 30 us).
-template <typename Body>
-__device__ __forceinline__ void region_walk(int nx, int Ry, int Rz, int RS, int plane, int ox,
-                                            int oy, int oz, int M, Body body) {
-    const FDiv fRz = fdiv_of(Rz);
-    const int M2 = M * M;
-    for (int e = threadIdx.x; e < Ry * Rz; e += blockDim.x) {
-        const int ry = fdiv(e, fRz), rz = e - ry * Rz;
-        int gx = wrap_index(ox, M);
-        int g = (gx * M + wrap_index(oy + ry, M)) * M + wrap_index(oz + rz, M);
-        int w = ry * RS + rz;
-#pragma unroll 4
-        for (int rx = 0; rx < nx; ++rx, w += plane) {
-            body(w, g);
-            g += M2;
-            if (++gx == M) {   // uniform
-                gx = 0;
-                g -= M2 * M;
-            }
-        }
-    }
-}
-
 // Spread of one tile (Eq. 3.5) into the fixed-point grid g64 (scale fxs =
 // 2^k): the n particles parts[0..n) of the tile.  The tile's region is
 // accumulated in shared memory as one 32-bit integer per point at the scale

@@ -60,7 +60,7 @@ cudaError_t launch_scatter(const T* xyz, const T* q, const KParams<T>& kp, const
                            int* perm, cudaStream_t s);
 template <typename T>
 cudaError_t launch_spread_tiled(const v4_t<T>* sorted, const int* tile_start, T* grid,
-                                const KParams<T>& kp, bool comp, cudaStream_t s);
+                                const KParams<T>& kp, bool comp, const Acc* acc, cudaStream_t s);
 template <typename T>
 cudaError_t launch_spread_direct(const v4_t<T>* sorted, T* grid, const KParams<T>& kp,
                                  cudaStream_t s);

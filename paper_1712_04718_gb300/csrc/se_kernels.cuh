@@ -445,6 +445,37 @@ k_scatter(const T* __restrict__ xyz, const T* __restrict__ q, const KParams<T> k
     }
 }
 
+// Walk over the points of a staged region, nx planes of Ry x Rz points (origin
+// (ox, oy, oz) on the grid, rows RS apart, planes `plane` apart in the region), by
+// the whole block: body(w, g) with the point's index in the region and its
+// wrapped index in the grid.  A thread keeps its (y, z) and runs over the planes,
+// so that a point costs two additions instead of two divisions and three
+// wraps (about 20 instructions, which were half of the tile gather's: 639 ->
+// 372 us for the 64-box ensemble at P = 10, 38 -> 31 us for 100 200 atoms at
+// P = 8; the spread's flush 383 -> 349 and 34 -> 30 us).  Ix: the type of the grid's
+// indices.
+template <typename Ix = int, typename Body>
+__device__ __forceinline__ void region_walk(int nx, int Ry, int Rz, int RS, int plane, int ox,
+                                            int oy, int oz, int M, Body body) {
+    const FDiv fRz = fdiv_of(Rz);
+    const Ix M2 = (Ix)M * M;
+    for (int e = threadIdx.x; e < Ry * Rz; e += blockDim.x) {
+        const int ry = fdiv(e, fRz), rz = e - ry * Rz;
+        int gx = wrap_index(ox, M);
+        Ix g = ((Ix)gx * M + wrap_index(oy + ry, M)) * M + wrap_index(oz + rz, M);
+        int w = ry * RS + rz;
+#pragma unroll 4
+        for (int rx = 0; rx < nx; ++rx, w += plane) {
+            body(w, g);
+            g += M2;
+            if (++gx == M) {   // uniform
+                gx = 0;
+                g -= M2 * M;
+            }
+        }
+    }
+}
+
 // Exact rounding error of the sum old + val as rounded by the atomic add
 // (two-sum; the atomic rounds to nearest even).
 template <typename T>
@@ -458,16 +489,34 @@ __device__ __forceinline__ T two_sum_err(T old, T val) {
 // a3: spread, shared-memory tiles.  One CTA per tile of `tile`^3 cells.  The
 // particles of the tile add their P^3 weights q c_g gx gy gz into the tile's
 // region ((tile + P - 1)^3 points) in shared memory; the region is then added
-// to the global grid, each nonzero point once per tile.  With COMP the
-// shared-memory sums are compensated: every add's rounding error (two-sum
-// against the value the atomic returned) goes to a second array, and the
-// region value flushed is hi + lo.  Regions larger than the shared-memory
-// budget are processed in slabs of `slab` x-planes.
+// to the global grid, each nonzero point once per tile.  With COMP a point has
+// two words, in one of two forms:
+//  - Integers, for tiles of at most kWordsMax particles: with 2^e > c_g max|q|
+//    over the tile's particles, hi counts units of 2^(e - K) and lo what its
+//    rounding leaves in units of 2^(e - K - K2), K = min(22, 30 - ceil(log2 n)),
+//    K2 = min(23, 31 - ceil(log2 n)), so that no sum can reach 2^31.  A weight is
+//    kept to 2^-(K + K2 + 1) of 2^e (2^-46 up to 256 particles, 2^-44 at
+//    kWordsMax, where FP32 weights carry 2^-24 of their own), both adds are
+//    native 32-bit shared atomics without a result, and the sums are exact.
+//  - Otherwise (crowded tiles, NaN or infinite input, scales near the ends of
+//    the FP32 range) compensated FP32 sums: every add's rounding error (two-sum
+//    against the value the atomic returned) goes to a second array.  FP32
+//    shared atomics are compare-and-swap loops, and each waits for its result.
+// The region value flushed is hi + lo, rounded once.  With the words in place of
+// the compensated sums (and region_walk in the flush) a whole evaluation of
+// 410 154 atoms at M = 135, P = 8 takes 425 us instead of 706 (this kernel had
+// 450 of them), one with ik forces of 21 642 atoms 140 instead of 174; errors
+// against 64-bit sums are unchanged (1.2e-5 and 5.2e-6, the FP32 positions').
+// kWordsMax: a water box has about 90 particles in a tile of edge 8 and 700 in
+// one of edge 16 at the finest; at 512 the words still keep 20 bits more than the weights.
+// Regions larger than the
+// shared-memory budget are processed in slabs of `slab` x-planes.
 // ---------------------------------------------------------------------------
+constexpr int kWordsMax = 512;
 template <typename T, int P, bool COMP>
 __global__ void __launch_bounds__(256)
 k_spread_tiled(const v4_t<T>* __restrict__ sorted, const int* __restrict__ tile_start,
-               T* __restrict__ grid, const KParams<T> kp, int slab) {
+               T* __restrict__ grid, const KParams<T> kp, int slab, const Acc* __restrict__ acc) {
     constexpr int D = pick_d(P), G = P / D, GPW = 32 / G;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T* hi = reinterpret_cast<T*>(smem_raw);
@@ -484,6 +533,34 @@ k_spread_tiled(const v4_t<T>* __restrict__ sorted, const int* __restrict__ tile_
     const int Rx = min(TT, M - t0x) + P - 1;
     const int plane = Ry * Rz;
     T* lo = hi + (size_t)slab * plane;
+
+    // the integer words' scales (words: uniform over the block)
+    bool words = false;
+    float S = 0.0f, S2 = 0.0f, Sinv = 0.0f;
+    if constexpr (COMP && sizeof(T) == 4) {
+        __shared__ float s_q[8];
+        const int n = pend - pbeg;
+        if (n <= kWordsMax && acc->nonfinite == 0) {   // uniform
+            float m = 0.0f;
+            for (int p = pbeg + threadIdx.x; p < pend; p += blockDim.x)
+                m = fmaxf(m, fabsf((float)sorted[p].w));
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+            if ((threadIdx.x & 31) == 0) s_q[threadIdx.x >> 5] = m;
+            __syncthreads();
+#pragma unroll
+            for (int w = 0; w < 8; ++w) m = fmaxf(m, s_q[w]);
+            const float B = m * (float)kp.qcg * 1.0001f;
+            if (B > 1e-20f && B < 1e20f) {
+                const int e = ilogbf(B) + 1, ln = n > 1 ? 32 - __clz(n - 1) : 0;
+                const int K = min(22, 30 - ln), K2 = min(23, 31 - ln);
+                words = true;
+                S = ldexpf(1.0f, K - e);
+                S2 = ldexpf(1.0f, K2);
+                Sinv = ldexpf(1.0f, e - K - K2);
+            }
+        }
+    }
 
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int gi = lane / G, k = lane - gi * G;
@@ -538,7 +615,15 @@ k_spread_tiled(const v4_t<T>* __restrict__ sorted, const int* __restrict__ tile_
                         for (int j = 0; j < D; ++j) {
                             const T val = wab * gz[j];
                             T* dst = base + j * G;
-                            if (COMP) {
+                            if (COMP && words) {
+                                // rounding to integers by adding 1.5 2^23
+                                const float t = fmaf((float)val, S, 12582912.0f);
+                                const float r = fmaf((float)val, S, -(t - 12582912.0f));   // exact
+                                const float t2 = fmaf(r, S2, 12582912.0f);
+                                atomicAdd(reinterpret_cast<int*>(dst), __float_as_int(t) - 0x4b400000);
+                                atomicAdd(reinterpret_cast<int*>(lo) + (dst - hi),
+                                          __float_as_int(t2) - 0x4b400000);
+                            } else if (COMP) {
                                 const T old = atomicAdd(dst, val);
                                 atomicAdd(lo + (dst - hi), two_sum_err(old, val));
                             } else {
@@ -550,19 +635,19 @@ k_spread_tiled(const v4_t<T>* __restrict__ sorted, const int* __restrict__ tile_
             }
         }
         __syncthreads();
-        const int ox = t0x - P / 2 + 1 + s0, oy = t0y - P / 2 + 1, oz = t0z - P / 2 + 1;
-        const FDiv fRz = fdiv_of(Rz), fRy = fdiv_of(Ry);
-        for (int e = threadIdx.x; e < nel; e += blockDim.x) {
+        region_walk<long long>(ns, Ry, Rz, Rz, plane, t0x - P / 2 + 1 + s0, t0y - P / 2 + 1,
+                               t0z - P / 2 + 1, M, [&](int e, long long g) {
             T val = hi[e];
-            if (COMP) val = add_rn(val, lo[e]);
-            if (val != T(0)) {
-                const int r = fdiv(e, fRz), rz = e - r * Rz;
-                const int rx = fdiv(r, fRy), ry = r - rx * Ry;
-                const int gx_ = wrap_index(ox + rx, M), gy_ = wrap_index(oy + ry, M),
-                          gz_ = wrap_index(oz + rz, M);
-                atomicAdd(grid + ((size_t)gx_ * M + gy_) * M + gz_, val);
+            if (COMP && words) {
+                const int h = __float_as_int((float)val), l = __float_as_int((float)lo[e]);
+                // (h 2^K2 + l) Sinv, rounded once but for the last bits of l
+                const float hf = (float)h;
+                val = fmaf(hf, S2, fmaf((float)(h - (int)hf), S2, (float)l)) * Sinv;
+            } else if (COMP) {
+                val = add_rn(val, lo[e]);
             }
-        }
+            if (val != T(0)) atomicAdd(grid + g, val);
+        });
         __syncthreads();
     }
 }

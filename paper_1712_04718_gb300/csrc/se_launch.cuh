@@ -39,7 +39,7 @@ cudaError_t launch_scatter(const T* xyz, const T* q, const KParams<T>& kp, const
 
 template <typename T, int P, bool COMP>
 cudaError_t spread_tiled_P(const v4_t<T>* sorted, const int* tile_start, T* grid,
-                           const KParams<T>& kp, cudaStream_t s) {
+                           const KParams<T>& kp, const Acc* acc, cudaStream_t s) {
     const size_t R = (size_t)kp.tile + P - 1;
     const size_t plane = R * R * sizeof(T) * (COMP ? 2 : 1);
     const int slab = (int)std::min(R, kSmemBudget / plane);
@@ -49,17 +49,17 @@ cudaError_t spread_tiled_P(const v4_t<T>* sorted, const int* tile_start, T* grid
                                          cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)kSmemBudget);
     if (e != cudaSuccess) return e;
-    k_spread_tiled<T, P, COMP><<<kp.ntiles, kThreads, bytes, s>>>(sorted, tile_start, grid, kp, slab);
+    k_spread_tiled<T, P, COMP><<<kp.ntiles, kThreads, bytes, s>>>(sorted, tile_start, grid, kp, slab, acc);
     return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t launch_spread_tiled(const v4_t<T>* sorted, const int* tile_start, T* grid,
-                                const KParams<T>& kp, bool comp, cudaStream_t s) {
+                                const KParams<T>& kp, bool comp, const Acc* acc, cudaStream_t s) {
     switch (kp.P) {
 #define SE_CASE(PP) \
-    case PP: return comp ? spread_tiled_P<T, PP, true>(sorted, tile_start, grid, kp, s) \
-                         : spread_tiled_P<T, PP, false>(sorted, tile_start, grid, kp, s);
+    case PP: return comp ? spread_tiled_P<T, PP, true>(sorted, tile_start, grid, kp, acc, s) \
+                         : spread_tiled_P<T, PP, false>(sorted, tile_start, grid, kp, acc, s);
         SE_FOR_EACH_P(SE_CASE)
 #undef SE_CASE
         default: return cudaErrorInvalidValue;
@@ -133,7 +133,7 @@ cudaError_t launch_gather(const v4_t<T>* sorted, const int* perm, const T* grid,
     template cudaError_t launch_scatter<T>(const T*, const T*, const KParams<T>&, const int*,    \
                                            const int*, const int*, v4_t<T>*, int*, cudaStream_t); \
     template cudaError_t launch_spread_tiled<T>(const v4_t<T>*, const int*, T*,                 \
-                                                const KParams<T>&, bool, cudaStream_t);         \
+                                                const KParams<T>&, bool, const Acc*, cudaStream_t);         \
     template cudaError_t launch_spread_direct<T>(const v4_t<T>*, T*, const KParams<T>&,         \
                                                  cudaStream_t);                                 \
     template cudaError_t launch_scale<T>(void*, const double*, int, T*, long long, double*,     \

@@ -101,7 +101,7 @@ extern "C" int se_spread_noalloc(const double* xyz, const double* q, int64_t N, 
     if (se::launch_scatter<double>(xyz, q, kp, slot, tile_of, tile_start, sorted, perm, s) !=
         cudaSuccess)
         return SE_ERR_CUDA;
-    if (N > 0 && se::launch_spread_tiled<double>(sorted, tile_start, H, kp, false, s) != cudaSuccess)
+    if (N > 0 && se::launch_spread_tiled<double>(sorted, tile_start, H, kp, false, nullptr, s) != cudaSuccess)
         return SE_ERR_CUDA;
     return SE_OK;
 }

@@ -647,7 +647,7 @@ int do_spread(se_plan* p, const void* xyz, const void* q) {
                 SE_CUDA(se::launch_spread_direct<T>((const V*)p->sorted, (T*)p->grid_spread, kp, p->stream));
             else
                 SE_CUDA(se::launch_spread_tiled<T>((const V*)p->sorted, p->tile_start, (T*)p->grid_spread,
-                                                   kp, p->prec == SE_FP32, p->stream));
+                                                   kp, p->prec == SE_FP32, p->acc, p->stream));
         }
     }
     timing_mark(p, 2);
