@@ -165,6 +165,8 @@ def unit_peaks(se, peaks):
     return {
         "fp32_fma_tflops": 152 * 128 * 2 * mhz * 1e6 / 1e12,
         "fp64_fma_tflops": 1.25,
+        # the double-precision sums run on split integers
+        "split_int_tflops": 152 * 64 * mhz * 1e6 * 2 / 3 / 1e12,
         "smem_atomic_gops": 152 * 32 * mhz * 1e6 / 1e9,
         "hbm_gbs": peaks.get("hbm_gbs", 6800.0),
         "hbm_source": "measured (MEASURED_PEAKS.json)" if "hbm_gbs" in peaks else "fallback",
@@ -320,7 +322,8 @@ def stage_work(w, prec, N, variant, tile=0):
         "spread": (("smem_atomic", float(N) * P ** 3, "k_fspread") if variant == 3 else
                    ("flop", 2.0 * N * P ** 3, "k_fdirect" if variant == 4 else "k_spread")),
         "gather": ("flop", 4.0 * N * P ** 3, "k_fgather" if variant == 3 and
-                   tile_gather_selected(N, M, P, tile) else "k_gather"),
+                   tile_gather_selected(N, M, P, tile) else
+                   ("k_gather_fx" if prec == "fp64" else "k_gather")),
         "bin": ("byte", N * (4 * ts + 8), "k_fbin" if variant == 3 else "k_bin"),
         "scatter": ("byte", N * (4 * ts + 4 * ts + 8 + 4), "k_scatter"),
     }
@@ -378,10 +381,11 @@ def roofline(kind, amount, kernel, us, prec, up, workload_name):
     elif kind == "flop":
         fp64 = prec == "fp64"
         r = {"bound": "alu", "unit": "TFLOP/s", "achieved": amount / secs / 1e12,
-             "peak": up["fp64_fma_tflops"] if fp64 else up["fp32_fma_tflops"],
-             "peak_source": ("GB300 nominal FP64 rate" if fp64 else
+             "peak": up["split_int_tflops"] if fp64 else up["fp32_fma_tflops"],
+             "peak_source": ("152 SMs x 64 32-bit integer multiply-adds into 64 bits/clock x max "
+                             "SM clock, three for each FP64 multiply-add of 2 flops" if fp64 else
                              "152 SMs x 128 FP32 lanes x 2 flops x max SM clock"),
-             "probe_peak": up["probe"]["fp64_fma_tflops" if fp64 else "fp32_fma_tflops"]}
+             "probe_peak": None if fp64 else up["probe"]["fp32_fma_tflops"]}
     else:
         r = {"bound": "hbm", "unit": "GB/s", "achieved": amount / secs / 1e9,
              "peak": up["hbm_gbs"], "peak_source": up["hbm_source"]}
