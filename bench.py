@@ -158,7 +158,9 @@ def unit_peaks(se, peaks):
     the shared-memory atomic rate are derived from unit counts and the
     maximum SM clock: 152 SMs x 128 FP32 lanes x 2 flops, and 152 SMs x 32
     banks (one 32-bit atomic per bank and clock); FP64 is GB300's nominal
-    1.25 TFLOP/s; HBM is the measured copy bandwidth.  The rates the
+    1.25 TFLOP/s, and for the sums over a particle's support, which run on
+    split integers, 152 SMs x 64 multiply-adds of 32-bit integers into 64
+    bits, three for each FP64 one; HBM is the measured copy bandwidth.  The rates the
     library's own probe kernels reach on this GPU (se_probe_peak) are given
     beside them."""
     mhz = float(peaks.get("sm_max_mhz", 2070.0))

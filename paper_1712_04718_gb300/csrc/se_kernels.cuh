@@ -508,9 +508,9 @@ __device__ __forceinline__ T two_sum_err(T old, T val) {
 // 450 of them), one with ik forces of 21 642 atoms 140 instead of 174; errors
 // against 64-bit sums are unchanged (1.2e-5 and 5.2e-6, the FP32 positions').
 // kWordsMax: a water box has about 90 particles in a tile of edge 8 and 700 in
-// one of edge 16 at the finest; at 512 the words still keep 20 bits more than the weights.
-// Regions larger than the
-// shared-memory budget are processed in slabs of `slab` x-planes.
+// one of edge 16 at the finest; at 512 the words still keep 20 bits more than
+// the weights.  Regions larger than the shared-memory budget are processed in
+// slabs of `slab` x-planes.
 // ---------------------------------------------------------------------------
 constexpr int kWordsMax = 512;
 template <typename T, int P, bool COMP>
