@@ -70,9 +70,9 @@ __device__ __forceinline__ double pow2i(int e) {
 }
 
 // Bits of the integer grid: a weight of the largest charge is below 2^bits, 56
-// but for crowded tiles, so that no grid point can reach 2^63: the weights of
-// the particles of a tile at distance d are at most e^{-beta d^2}, and summed
-// over all tiles at most crowd times the fullest tile's count (fx_params).
+// but for crowded tiles, so that no grid point can reach 2^63: all tiles together
+// give a point at most crowd times the fullest tile's count of such weights
+// (tile_crowd, which takes the tiles as they are cut, the narrow last ones too).
 __device__ __forceinline__ int grid_bits(const Acc* acc, const FxParams& fp) {
     const int n = min(fp.kp.N, __float2int_ru(fp.crowd * (float)acc->tile_max));   // saturates
     return min(56, 63 - (n > 1 ? 32 - __clz(n - 1) : 0));

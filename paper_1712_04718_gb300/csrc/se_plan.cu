@@ -88,6 +88,7 @@ struct se_plan {
     int* fx_cells = nullptr;
     int* fx_top = nullptr;
     double fx_gbound = 0.0;
+    double fx_crowd = 0.0;               // tile_crowd
     cudaStream_t fft_stream = nullptr;   // stream the FFT plans were last given
     bool fft_stream_set = false;
     void* fx_split = nullptr;
@@ -330,6 +331,28 @@ std::vector<double> green_table(const se_plan* p) {
     return g;
 }
 
+// What a grid point receives at most, in units of the weight of the largest
+// charge, if every tile holds one particle: the particles of a tile at distance
+// d (grid units, per dimension) weigh at most e^{-beta d^2}, so it is the cube of
+// the largest sum over the tiles of one dimension.  Two tiles meet at a face
+// point and the others are an edge or more away, except where the last tile is
+// narrow (M mod edge cells wide): there three lie within its width.
+double tile_crowd(const se_plan* p) {
+    const double beta = p->alpha * p->h * p->h;
+    double most = 0.0;
+    for (int x = 0; x < p->M; ++x) {
+        double sum = 0.0;
+        for (int a = 0; a < p->M; a += p->tile) {
+            const int b = std::min(a + p->tile, p->M);
+            const int d = x < a ? std::min(a - x, x + p->M - b)
+                                : (x > b ? std::min(x - b, a + p->M - x) : 0);
+            if (2 * d <= p->P + 2) sum += exp(-beta * d * d);   // farther ones do not reach
+        }
+        most = std::max(most, sum);
+    }
+    return most * most * most * (1.0 + 1e-6);
+}
+
 int prepare(se_plan* p) {
     int dev = 0;
     SE_CUDA(cudaGetDevice(&dev));
@@ -391,6 +414,7 @@ int prepare(se_plan* p) {
     }
     std::vector<double> g = green_table(p);
     if (p->prec == SE_FP64) {
+        p->fx_crowd = tile_crowd(p);
         // sum of G over the whole spectrum: the half spectrum's inner planes twice
         double sum = 0.0;
         const int Mh = p->M / 2 + 1;
@@ -517,11 +541,7 @@ se::FxParams fx_params(const se_plan* p) {
     // the sums over y, x and z in bits, each kept below 63 (a margin of 2^-6
     // covers the rounding of the factors and of the bound)
     const double gs = log2(std::max(g, dg)) + 1.0 / 64.0, top = 63.0;
-    // the tiles' largest weights at a point, summed over the tiles: at a face,
-    // distances 0, 0, T, T, 2T, 2T, ... per dimension
-    double k = 0.0;
-    for (int i = 0; i * p->tile <= p->P; ++i) k += 2.0 * exp(-beta * i * p->tile * i * p->tile);
-    f.crowd = (float)(k * k * k * (1.0 + 1e-6));
+    f.crowd = (float)p->fx_crowd;
     f.gbound = p->fx_gbound;
     const double M3 = (double)p->M * p->M * p->M;   // fx_gbound^2 M^3 = sum_k G / M^3
     f.gbound1 = p->fx_gbound * p->fx_gbound * M3 * f.kp.qcg * g * g * g;

@@ -1,0 +1,70 @@
+"""Limits of the double-precision integer spread and gather: what one grid
+point can receive where the last tile is narrow, charges near the ends of the
+FP64 range, systems whose charges crowd or differ so much that the integer
+grid's quantum would show, rounding without a preferred sign, ranges of
+particles, and the memory that a plan takes.
+
+Tolerances as the other FP64 comparisons (1e-12 for grids, 5e-12 for particle
+outputs) unless a test says otherwise."""
+import math
+
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_1712_04718_gb300 import se, systems
+from parity import assert_close
+
+pytestmark = pytest.mark.gpu
+
+TOL = 1e-12
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    import __graft_entry__
+    __graft_entry__.build()
+    torch.cuda.set_device(0)
+
+
+def _xi(L, M, P, most=0.7):
+    return min(4.0, math.sqrt(most * 0.95 ** 2 * math.pi * M * M / (P * L * L)))
+
+
+def _dev(a):
+    return torch.tensor(a, device="cuda", dtype=torch.float64)
+
+
+def _evaluate(x, q, L, xi, M, P, **kw):
+    plan = se.Plan(len(q), L, xi, M, P, precision="fp64", **kw)
+    xd, qd = _dev(x), _dev(q)
+    plan.spread(xd, qd)
+    H = plan.copy_grid(0).cpu().numpy()
+    F, phi = torch.empty_like(xd), torch.empty_like(qd)
+    E = torch.zeros(1, dtype=torch.float64, device="cuda")
+    plan.evaluate(xd, qd, F, phi, E)
+    torch.cuda.synchronize()
+    plan.close()
+    return H, F.cpu().numpy(), phi.cpu().numpy(), E.item()
+
+
+@pytest.mark.parametrize("M,P,tile,c", [(33, 24, 8, 10), (33, 8, 8, 14), (41, 8, 8, 60),
+                                        (57, 16, 8, 30), (34, 8, 8, 15), (26, 24, 5, 10),
+                                        (32, 8, 8, 60)])
+def test_cluster_at_the_narrow_last_tile(M, P, tile, c):
+    """c equal charges in each of the 27 tiles round the box's corner, within a
+    cell of it where the last tile is one cell wide: every one of them reaches
+    the corner's grid point with nearly its whole weight."""
+    L = 2.0
+    h = L / M
+    a = np.array([1e-3, M - 1e-3, (M - M % tile if M % tile else M - 1) - 1e-3]) * h
+    x = np.stack(np.meshgrid(a, a, a, indexing="ij"), -1).reshape(-1, 3).repeat(c, axis=0)
+    q = np.ones(27 * c)      # not neutral: the k = 0 mode is dropped
+    xi = _xi(L, M, P)
+    H, F, phi, E = _evaluate(x, q, L, xi, M, P, tile=tile)
+    r = oracle.se_kspace(x, q, L, xi, M, P, cell_mode=64, grids=True)
+    assert_close(H, r["H"], TOL, label="spread grid")
+    assert_close(phi, r["phi"], 5 * TOL, label="phi")
+    assert_close(F, r["F"], 5 * TOL, label="F", q=q)
+    assert abs(E - r["E"]) < 5 * TOL * abs(r["E"])
