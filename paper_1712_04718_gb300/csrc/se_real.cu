@@ -181,10 +181,10 @@ k_rs_scatter(const T* __restrict__ xyz, const T* __restrict__ q, int N, T L, T i
     v.w = q[i];
     sorted[p] = v;
     if constexpr (sizeof(T) == 8) {   // the copy that the distance test of k_rs_pairs64 reads
-        se::f4 f;
-        f.x = (float)v.x;
-        f.y = (float)v.y;
-        f.z = (float)v.z;
+        se::f4 f;                     // in units of L: its squares are in range whatever the units
+        f.x = (float)(v.x * invL);
+        f.y = (float)(v.y * invL);
+        f.z = (float)(v.z * invL);
         f.w = 0.0f;
         sorted_f[p] = f;
     }
@@ -435,8 +435,8 @@ k_rs_pairs(const se::f4* __restrict__ sorted, const int* __restrict__ start,
 // of its pairs and by nothing else; the design spends as few as it can:
 //
 //  - The distance test, which 73 % of the candidates fail on a water box, is
-//    made in FP32 with a bound wide enough for every FP32 rounding on the way
-//    (rs_run); the pairs that pass are tested again in FP64, as before, so
+//    made in FP32, on positions in units of L, with a bound wide enough for
+//    every FP32 rounding on the way (rs_run); the pairs that pass are tested again in FP64, as before, so
 //    the set of pairs that are summed is the same.
 //  - erfc(x)/x and (2/sqrt(pi) e^{-x^2} + erfc(x)/x)/x^2 are both smooth
 //    functions of v = x^2 = xi^2 r^2 alone, which needs no square root.  They
@@ -509,7 +509,6 @@ k_rs_pairs64(const se::d4* __restrict__ sorted, const se::f4* __restrict__ sorte
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (nh > 0) stencil_ranges(start, nc, K, cx, cy, cz, s_b0, s_off, s_sh);   // per block
     const int total = nh > 0 ? s_off[W3] : 0;
-    const float Lf = (float)L;
     const double xi2 = xi * xi;
     const long long rc2_bits = __double_as_longlong(rc2);
     unsigned short* q = s_q[warp];
@@ -563,7 +562,7 @@ k_rs_pairs64(const se::d4* __restrict__ sorted, const se::f4* __restrict__ sorte
                     const int k = stencil_cell(s_off, W3, c0 + t);
                     const int p = s_b0[k] + c0 + t - s_off[k];
                     nb[t] = image_of(sorted[p], s_sh[k], L);
-                    nf[t] = image_of(sorted_f[p], s_sh[k], Lf);
+                    nf[t] = image_of(sorted_f[p], s_sh[k], 1.0f);
                 }
                 __syncthreads();
             }
@@ -707,7 +706,7 @@ struct se_real {
     int* slot = nullptr;
     int* perm = nullptr;
     void* sorted = nullptr;
-    se::f4* sorted_f = nullptr;      // FP64: the positions in FP32
+    se::f4* sorted_f = nullptr;      // FP64: the positions / L in FP32
     double2* table = nullptr;        // FP64: the pair functions (vtable)
     double* partials = nullptr;
     unsigned* ticket = nullptr;
@@ -779,12 +778,12 @@ int rs_run(se_real* r, const void* xyz, const void* q, void* F, void* phi, doubl
     k_rs_scatter<T><<<nb, kThreads, 0, s>>>((const T*)xyz, (const T*)q, N, L, invL, r->cell_of,
                                             r->slot, r->start, (V*)r->sorted, r->sorted_f, r->perm);
     if constexpr (sizeof(T) == 8) {
-        // The bound of the FP32 distance test.  A position rounded to FP32 is
-        // off by at most L 2^-24, an image of it (the shift by L rounded, and
-        // the sum) and a difference of two by at most e = 8 L 2^-24 in all per
-        // axis, so a pair within r_c has an FP32 distance within r_c + 2 e;
+        // The bound of the FP32 distance test, in units of L.  A position
+        // rounded to FP32 is off by at most 2^-24, an image of it (the sum
+        // with +-1) and a difference of two by at most e = 8 2^-24 in all per
+        // axis, so a pair within r_c has an FP32 distance within r_c / L + 2 e;
         // its square is formed with a relative error below 2^-21.
-        const double e = 8.0 * r->L / 16777216.0, rf = r->rc + 2.0 * e;
+        const double e = 8.0 / 16777216.0, rf = r->rc / r->L + 2.0 * e;
         const float rc2_f = (float)(rf * rf * (1.0 + 1.0 / 1048576.0));
         const int bytes = kCap64 * (int)(sizeof(se::d4) + sizeof(se::f4));
         if (cudaFuncSetAttribute(k_rs_pairs64, cudaFuncAttributeMaxDynamicSharedMemorySize,
