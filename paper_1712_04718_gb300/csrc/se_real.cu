@@ -484,6 +484,14 @@ __device__ __forceinline__ double warp_sum4(double a, double b, double c, double
     return z;
 }
 
+// The pair sums of potential and force are kept in units of s and s^3: xi, as the
+// table has them, or 1 where every pair is nearer than the table begins (bare:
+// xi r_c below 2^-5/2), so that a small xi r needs no power of itself.
+struct PairScales {
+    double xi, c2xi, s;   // c2xi = 2 xi / sqrt(pi)
+    bool bare;
+};
+
 constexpr int kPair64Warps = 6;
 constexpr int kCap64 = 2048;        // staged candidates (96 KB: two CTAs per SM)
 constexpr int kTest64 = 128;        // candidates tested per step
@@ -492,7 +500,7 @@ constexpr int kQueue64 = kTest64 + 32;
 __global__ void __launch_bounds__(32 * kPair64Warps)
 k_rs_pairs64(const se::d4* __restrict__ sorted, const se::f4* __restrict__ sorted_f,
              const int* __restrict__ start, const int* __restrict__ perm, int nc, int K, double L,
-             double rc2, float rc2_f, double xi, double kc, const double2* __restrict__ table,
+             double rc2, float rc2_f, const PairScales sc, double kc, const double2* __restrict__ table,
              double* __restrict__ phi, double* __restrict__ F, int accumulate,
              double* __restrict__ partials, unsigned* ticket, double* E_out) {
     extern __shared__ __align__(32) unsigned char smem_raw[];
@@ -509,7 +517,7 @@ k_rs_pairs64(const se::d4* __restrict__ sorted, const se::f4* __restrict__ sorte
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (nh > 0) stencil_ranges(start, nc, K, cx, cy, cz, s_b0, s_off, s_sh);   // per block
     const int total = nh > 0 ? s_off[W3] : 0;
-    const double xi2 = xi * xi;
+    const double xi2 = sc.xi * sc.xi;
     const long long rc2_bits = __double_as_longlong(rc2);
     unsigned short* q = s_q[warp];
     double e_loc = 0.0;
@@ -546,7 +554,8 @@ k_rs_pairs64(const se::d4* __restrict__ sorted, const se::f4* __restrict__ sorte
                     g = fma(g, t, w.y);
                 }
             } else {   // very close or very far pairs
-                pair_terms(v, rsqrt(v), 1.0, 1.1283791670955126, f, g);
+                if (sc.bare) pair_terms(r2, rsqrt(r2), sc.xi, sc.c2xi, f, g);
+                else pair_terms(v, rsqrt(v), 1.0, 1.1283791670955126, f, g);
             }
             ph += n.w * f;
             const double fq = n.w * g;
@@ -603,11 +612,11 @@ k_rs_pairs64(const se::d4* __restrict__ sorted, const se::f4* __restrict__ sorte
             const int o = perm[h0 + pass0 + warp], k = lane >> 3;
             if ((lane & 7) == 0) {
                 if (k == 0) {
-                    const double pm = kc * (xi * sum - 1.1283791670955126 * xi * me.w);
+                    const double pm = kc * (sc.s * sum - sc.c2xi * me.w);
                     if (phi) phi[o] = accumulate ? phi[o] + pm : pm;
                     e_loc += me.w * pm;
                 } else if (F) {
-                    const double f = kc * me.w * (xi * xi2 * sum);
+                    const double f = kc * me.w * (sc.s * sum * sc.s * sc.s);
                     double* dst = F + 3 * (size_t)o + (k - 1);
                     *dst = accumulate ? *dst + f : f;
                 }
@@ -785,13 +794,16 @@ int rs_run(se_real* r, const void* xyz, const void* q, void* F, void* phi, doubl
         // its square is formed with a relative error below 2^-21.
         const double e = 8.0 / 16777216.0, rf = r->rc / r->L + 2.0 * e;
         const float rc2_f = (float)(rf * rf * (1.0 + 1.0 / 1048576.0));
+        const bool bare = r->xi * r->rc < 0.17;
+        const PairScales sc = {r->xi, 2.0 * r->xi / sqrt(3.14159265358979323846),
+                               bare ? 1.0 : r->xi, bare};
         const int bytes = kCap64 * (int)(sizeof(se::d4) + sizeof(se::f4));
         if (cudaFuncSetAttribute(k_rs_pairs64, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  bytes) != cudaSuccess)
             return SE_ERR_CUDA;
         k_rs_pairs64<<<r->ncells, 32 * kPair64Warps, bytes, s>>>(
             (const V*)r->sorted, r->sorted_f, r->start, r->perm, nc, r->K, L, r->rc * r->rc, rc2_f,
-            r->xi, r->kc, r->table, (T*)phi, (T*)F, acc, r->partials, r->ticket, E);
+            sc, r->kc, r->table, (T*)phi, (T*)F, acc, r->partials, r->ticket, E);
     } else {
         const int cap = (int)(kNbSmem / sizeof(V));
         if (cudaFuncSetAttribute(k_rs_pairs, cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -66,3 +66,12 @@ def test_positions_that_differ_by_a_rounding_of_the_test():
         x += [a, a + rc * (1 + k * 2.0 ** -23) * d / np.linalg.norm(d)]
     x = np.array(x)
     _check(x, np.ones(len(x)), L, xi, rc)
+
+
+@pytest.mark.parametrize("xi", [1e-8, 1e-60, 1e-103, 1e-110, 1e-155, 1e-200])
+def test_bare_coulomb_limit(xi):
+    """xi r far below one: erfc(xi r)/r is 1/r."""
+    L, rc = 3.0, 1.0
+    rng = np.random.default_rng(9)
+    x = L * rng.random((200, 3))
+    _check(x, rng.uniform(0.5, 1.0, 200), L, xi, rc)
