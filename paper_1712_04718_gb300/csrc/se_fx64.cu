@@ -61,10 +61,12 @@ k_fx_fold(const long long* __restrict__ g, int Mp, int p0, const FxParams fp,
 // small that the energy leaves the normal range (beyond about 1e+-145) take
 //   |Ht(x)| <= sum_k G/M^3 sum_x |H(x)|,  sum_x |H| <= sum_n |q_n| c_g W^3
 // instead, W a bound of the sum of a window's factors (gbound1).  Block 0 leaves
-// the biased exponent E + 1022 in *top.
+// the biased exponent E + 1022 in *top.  Inf and NaN values (finite charges whose
+// grid or transform overflowed) have no place in the split grid: they set
+// acc->overflow, and the gather gives NaN.
 __global__ void __launch_bounds__(256)
 k_grid_split(const double* __restrict__ grid, int M, int Mp, int p0, double gbound,
-             double gbound1, const Acc* __restrict__ acc, int* __restrict__ top, int hb, int2* __restrict__ out) {
+             double gbound1, Acc* acc, int* __restrict__ top, int hb, int2* __restrict__ out) {
     __shared__ int s_top;
     if (threadIdx.x == 0) {
         const double e = acc->e_grid;
@@ -81,6 +83,7 @@ k_grid_split(const double* __restrict__ grid, int M, int Mp, int p0, double gbou
         for (int z = lane; z < Mp; z += 32) {
             const long long b = __double_as_longlong(__ldg(src + wrap_index(z - p0, M)));
             const int e = (int)(b >> 52) & 0x7ff;
+            if (e == 0x7ff) acc->overflow = 1u;
             const long long mant = (b & 0xfffffffffffffLL) | (e ? 1LL << 52 : 0LL);   // < 2^53
             // |value| = mant 2^(max(e,1) - 1075); hb + 32 bits below 2^E, E = etop - 1022
             const int sh = max(0, etop - max(e, 1));

@@ -260,7 +260,8 @@ k_gather_fx(const int4* __restrict__ fac, const int* __restrict__ cells,
     const int Mp = kp.M + P - 1;
     // the grid's units 2^(E - hb); the sums are scaled by 2^30 per window and
     // cut by 2^(32 + e1) and 2^(32 + e2); NaN where an input was NaN or infinite
-    const double unit = acc->nonfinite
+    // or the grid overflowed
+    const double unit = acc->nonfinite | acc->overflow
                             ? CUDART_NAN
                             : pow2i(top[0] - 1022 - fp.hb - 26 + fp.e1 + fp.e2);
     const double gsc = adj ? __ldg(adj) : 1.0;

@@ -46,7 +46,7 @@ struct Acc {
     float fx_scale, fx_inv;  // 2^fx_shift and 2^-fx_shift
     double qscale, qunit;    // 1 / max|q| (a little less) and its inverse (k_bin)
     int tile_max;            // particles of the fullest tile (k_bin)
-    int pad;
+    unsigned int overflow;   // the transformed grid has Inf or NaN values (k_grid_split)
 };
 
 // launchers (se_kernels_*.cu)

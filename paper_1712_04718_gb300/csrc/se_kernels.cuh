@@ -423,6 +423,7 @@ k_bin(const T* __restrict__ xyz, const T* __restrict__ q, const KParams<T> kp,
     if (threadIdx.x == blockDim.x - 1) {
         tile_start[n] = run;
         acc->tile_max = s_tmax;
+        acc->overflow = 0u;
     }
 }
 

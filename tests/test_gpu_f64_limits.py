@@ -68,3 +68,19 @@ def test_cluster_at_the_narrow_last_tile(M, P, tile, c):
     assert_close(phi, r["phi"], 5 * TOL, label="phi")
     assert_close(F, r["F"], 5 * TOL, label="F", q=q)
     assert abs(E - r["E"]) < 5 * TOL * abs(r["E"])
+
+
+def test_grid_beyond_the_range_gives_nan():
+    """Finite charges whose grid or transform overflows: no finite number."""
+    L, xi, M, P = 2.0, 3.0, 24, 8
+    x, q = systems.uniform_charges(200, L, seed=5)
+    plan = se.Plan(len(q), L, xi, M, P, precision="fp64")
+    xd = _dev(x)
+    F, phi = torch.empty_like(xd), torch.empty(len(q), dtype=torch.float64, device="cuda")
+    for scale in (1e306, 1e307):
+        plan.evaluate(xd, _dev(q * scale), F, phi)
+        assert not phi.isfinite().any() and not F.isfinite().any()
+    plan.evaluate(xd, _dev(q), F, phi)   # and the next call is as any other
+    r = oracle.se_kspace(x, q, L, xi, M, P, cell_mode=64)
+    assert_close(phi.cpu().numpy(), r["phi"], 5 * TOL, label="phi")
+    plan.close()
