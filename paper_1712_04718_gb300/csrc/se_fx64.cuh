@@ -69,6 +69,10 @@ __device__ __forceinline__ double pow2i(int e) {
     return e >= -1074 ? __longlong_as_double(1LL << (e + 1074)) : 0.0;
 }
 
+// Scales below 2^kTinyExp are taken 2^kTinyShift times larger and the results
+// made smaller at the end, so that no scale is subnormal.
+constexpr int kTinyExp = -850, kTinyShift = 200;
+
 // Bits of the integer grid: a weight of the largest charge is below 2^bits, 56
 // but for crowded tiles, so that no grid point can reach 2^63: all tiles together
 // give a point at most crowd times the fullest tile's count of such weights
@@ -261,9 +265,10 @@ k_gather_fx(const int4* __restrict__ fac, const int* __restrict__ cells,
     // the grid's units 2^(E - hb); the sums are scaled by 2^30 per window and
     // cut by 2^(32 + e1) and 2^(32 + e2); NaN where an input was NaN or infinite
     // or the grid overflowed
-    const double unit = acc->nonfinite | acc->overflow
-                            ? CUDART_NAN
-                            : pow2i(top[0] - 1022 - fp.hb - 26 + fp.e1 + fp.e2);
+    const int ue = top[0] - 1022 - fp.hb - 26 + fp.e1 + fp.e2;
+    const bool tiny = ue < kTinyExp;
+    const double unit = acc->nonfinite | acc->overflow ? CUDART_NAN
+                                                       : pow2i(ue + (tiny ? kTinyShift : 0));
     const double gsc = adj ? __ldg(adj) : 1.0;
     const double u_phi = unit * kp.phi_scale;
     const double u_F = unit * kp.F_scale * pow2i(fp.sd) * (adj ? -gsc : 1.0);
@@ -351,7 +356,8 @@ k_gather_fx(const int4* __restrict__ fac, const int* __restrict__ cells,
             for (int j = 0; j < (4 + P - 1) / P; ++j) {
                 const int c = k + j * P;
                 if (c > 3) break;
-                const double w = (double)mine[j] * (c == 0 ? u_phi : u_F);
+                double w = (double)mine[j] * (c == 0 ? u_phi : u_F);
+                if (tiny) w *= pow2i(-kTinyShift);   // uniform
                 if (c == 0) {
                     if (phi) phi[orig] = w * gsc;
                     e_loc += qq * w;

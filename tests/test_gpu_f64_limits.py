@@ -84,3 +84,15 @@ def test_grid_beyond_the_range_gives_nan():
     r = oracle.se_kspace(x, q, L, xi, M, P, cell_mode=64)
     assert_close(phi.cpu().numpy(), r["phi"], 5 * TOL, label="phi")
     plan.close()
+
+
+@pytest.mark.parametrize("scale", [1e-300, 1e-295, 1e295, 1e300])
+def test_charges_near_the_ends_of_the_range(scale):
+    """Results keep their digits where products of two scales would be
+    subnormal or overflow."""
+    L, xi, M, P = 2.0, 3.0, 24, 8
+    x, q = systems.uniform_charges(200, L, seed=5)
+    H, F, phi, _ = _evaluate(x, q * scale, L, xi, M, P)
+    r = oracle.se_kspace(x, q, L, xi, M, P, cell_mode=64, grids=True)
+    assert_close(H / scale, r["H"], TOL, label="spread grid")
+    assert_close(phi / scale, r["phi"], 5 * TOL, label="phi")
