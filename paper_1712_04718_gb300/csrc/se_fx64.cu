@@ -19,43 +19,49 @@ SE_P_LIST(SE_FX_EXTERN)
 namespace {
 
 // The padded integer grid (units of 2^-grid_bits of the largest charge, times
-// c_g) -> FP64: every grid point is the sum of its images.  A warp takes a row
-// (x, y).  The scaling step clears the integer grid: clearing what was read here
+// c_g) -> FP64: every grid point is the sum of its images.  For FP64 sums the grid
+// holds FP64 numbers in units of the largest charge's power of two.  A warp takes
+// a row (x, y).  The scaling step clears the grid: clearing what was read here
 // made the loads wait for the stores (113 us instead of 16 for 119^3 points).
 __global__ void __launch_bounds__(256)
 k_fx_fold(const long long* __restrict__ g, int Mp, int p0, const FxParams fp,
           const Acc* __restrict__ acc, double* __restrict__ grid) {
+    const int bits = grid_bits(acc, fp);
     const bool tiny = acc->qunit < 0x1p-850;   // 2^kTinyExp
+    const int up = tiny ? kTinyShift : 0;
+    const double base = bits > 0 ? acc->qunit * pow2i(up - bits)
+                                 : pow2i(((__double2hiint(acc->qunit) >> 20) & 0x7ff) - 1021 + up);
     // NaN or infinite input: NaN results
-    const double unit = acc->nonfinite ? CUDART_NAN
-                                       : fp.kp.qcg * (acc->qunit * pow2i((tiny ? kTinyShift : 0) -
-                                                                         grid_bits(acc, fp)));
+    const double unit = acc->nonfinite ? CUDART_NAN : fp.kp.qcg * base;
     const int M = fp.kp.M, warps = gridDim.x * (blockDim.x >> 5), lane = threadIdx.x & 31;
     // the images of index i: i + p0, and one more M above or below (P <= M)
     auto other = [&](int i) { return i <= p0 ? i + p0 + M : (i >= M - p0 ? i + p0 - M : -1); };
-    auto row = [&](int r, auto finish) {
-        const int x = r / M, y = r - x * M;
-        const int xo = other(x), yo = other(y);
-        for (int z = lane; z < M; z += 32) {
-            const int zo = other(z);
-            long long v = 0;
+    auto rows = [&](auto zero, auto value, auto finish) {
+        for (int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); r < M * M; r += warps) {
+            const int x = r / M, y = r - x * M;
+            const int xo = other(x), yo = other(y);
+            for (int z = lane; z < M; z += 32) {
+                const int zo = other(z);
+                auto v = zero;
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int px = j & 1 ? xo : x + p0, py = j & 2 ? yo : y + p0;
-                if (px < 0 || py < 0) continue;   // uniform over the warp
-                const long long* s = g + ((size_t)px * Mp + py) * Mp;
-                v += __ldg(s + z + p0);
-                if (zo >= 0) v += __ldg(s + zo);
+                for (int j = 0; j < 4; ++j) {
+                    const int px = j & 1 ? xo : x + p0, py = j & 2 ? yo : y + p0;
+                    if (px < 0 || py < 0) continue;   // uniform over the warp
+                    const long long* s = g + ((size_t)px * Mp + py) * Mp;
+                    v += value(__ldg(s + z + p0));
+                    if (zo >= 0) v += value(__ldg(s + zo));
+                }
+                grid[(size_t)r * M + z] = finish((double)v * unit);
             }
-            grid[(size_t)r * M + z] = finish((double)v * unit);
         }
     };
-    const int r0 = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (!tiny) {   // the branch outside the loops: within them it cost 6 us of 50 for 135^3 points
-        for (int r = r0; r < M * M; r += warps) row(r, [](double w) { return w; });
-    } else {
-        for (int r = r0; r < M * M; r += warps) row(r, [](double w) { return w * pow2i(-kTinyShift); });
-    }
+    // the branch outside the loops: within them it cost 6 us of 50 for 135^3 points
+    auto word = [](long long v) { return v; };
+    auto real = [](long long v) { return __longlong_as_double(v); };
+    auto down = [up](double w) { return w * pow2i(-up); };
+    if (bits == 0) rows(0.0, real, down);
+    else if (tiny) rows(0LL, word, down);
+    else rows(0LL, word, [](double w) { return w; });
 }
 
 // The grid split in units of 2^(E - hb), every |value| < 2^E, by integer

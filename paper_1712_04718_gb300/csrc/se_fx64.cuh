@@ -77,16 +77,43 @@ constexpr int kTinyExp = -850, kTinyShift = 200;
 // but for crowded tiles, so that no grid point can reach 2^63: all tiles together
 // give a point at most crowd times the fullest tile's count of such weights
 // (tile_crowd, which takes the tiles as they are cut, the narrow last ones too).
+// 0: the grid is summed in FP64, because the quantum 2^-bits is coarser than
+// 2^-kFxMinBits of the mean charge's largest weight.  FP64 sums keep 53 bits of
+// every weight however many meet in a tile and however large the largest charge
+// is, but FP64 reductions are slower than integer ones: 21 642 atoms, M = 52,
+// P = 8: 64 -> 68 us for all steps of the spread, M = 96, P = 24: 403 -> 664 (and
+// 226 and 981 with the FP64 tiles of before).  Relative error of the potentials
+// against extended precision, FP64 sums / integers at the bits in brackets: 20 000
+// charges of both signs in one place (P = 8) 3e-15 / 1.4e-12 (45), 2 000 1e-15 /
+// 2.8e-14 (49), 250 5e-16 / 1.1e-15 (53), 100 6e-16 / 8e-16 (54); one charge of 1e8
+// among 5 000 of 1 3e-16 / 1.8e-14 (52 for the large one); a water box 2.4e-15 /
+// 3.0e-15 (55).
+constexpr int kFxMinBits = 54;
 __device__ __forceinline__ int grid_bits(const Acc* acc, const FxParams& fp) {
     const int n = min(fp.kp.N, __float2int_ru(fp.crowd * (float)acc->tile_max));   // saturates
-    return min(56, 63 - (n > 1 ? 32 - __clz(n - 1) : 0));
+    const int bits = min(56, 63 - (n > 1 ? 32 - __clz(n - 1) : 0));
+    return acc->qmean >= __int_as_float((127 + kFxMinBits - bits) << 23) ? bits : 0;
+}
+
+// q as +-[1/4, 1/2) times 2^(field - 1021), field the biased exponent (below 1
+// for subnormal numbers); q = 0 gives 0.
+__device__ __forceinline__ double split_exponent(double q, int* field) {
+    int sub = 0;
+    if (((__double2hiint(q) >> 20) & 0x7ff) == 0) {
+        q *= 0x1p54;
+        sub = 54;
+    }
+    const int hi = __double2hiint(q);
+    *field = ((hi >> 20) & 0x7ff) - sub;
+    return q == 0.0 ? q : __hiloint2double((hi & 0x800fffff) | (1021 << 20), __double2loint(q));
 }
 
 // One thread per particle and dimension (dimension-major, so that a warp has
 // one).  fac[r][d][a] = (g hi, g lo, dg hi, dg lo) scaled by 2^30 and 2^(30 - sd):
 // the window and its derivative's offset factor dz g, dz = a - (P-1)/2 - u, at
 // support point a; xq[r][a] = q / max|q| times the x factor, scaled by
-// 2^(grid_bits - 27); r = position in tile order - c0.  Only particles with
+// 2^(grid_bits - 27), or for FP64 sums the charge's significand (split_exponent)
+// times the x factor, scaled by 2^30; r = position in tile order - c0.  Only particles with
 // c0 <= position < c1 get factors.  dz is split too (hi scaled by 2^26, one lo
 // for all a), so that dg costs integer operations only.
 // Bound by the FP64 pipe: two exponentials, a reciprocal and two operations a
@@ -116,7 +143,10 @@ k_scatter_fx(const double* __restrict__ xyz, const double* __restrict__ q, const
             qp = q[i];
             sorted[4 * (size_t)dst + 3] = qp;
             perm[dst] = i;
-            qp *= acc->qscale * pow2i(grid_bits(acc, fp) - 57);
+            const int bits = grid_bits(acc, fp);
+            int field;
+            if (bits > 0) qp *= acc->qscale * pow2i(bits - 57);
+            else qp = split_exponent(qp, &field);
         }
         if (dst < c0 || dst >= c1) continue;
         const double u = offset_of(x, c, kp.invh, fp.invh_lo);
@@ -169,16 +199,23 @@ constexpr int kFxThreads = 128;
 // an integer in units of 2^-3 of the grid's.  Particles come in tile order, but
 // nothing depends on it.
 // Bound by the L2's 64-bit reductions (about 2.4 lanes per clock and SM).
+// For FP64 sums (grid_bits) W, an integer of 2^-60 of the particle's own charge,
+// goes as an FP64 number in units of the largest charge's power of two to the
+// same grid, as FP64 reductions.
 template <int P>
 __global__ void __launch_bounds__(kFxThreads)
 k_spread_fx(const int4* __restrict__ fac, const int2* __restrict__ xq,
-            const int* __restrict__ cells, unsigned long long* __restrict__ g64, int Mp, int c0,
-            int c1) {
+            const int* __restrict__ cells, const double* __restrict__ sorted,
+            unsigned long long* __restrict__ g64, const FxParams fp, const Acc* __restrict__ acc,
+            int c0, int c1) {
     constexpr int GPW = kFxGPW<P>, BC = kFxRows<P>;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int gi = lane / P, k = lane - gi * P;
     if (gi >= GPW) return;
+    const int Mp = fp.kp.M + P - 1;
     const int per = (kFxThreads / 32) * GPW;
+    const bool words = grid_bits(acc, fp) > 0;   // uniform over the grid
+    const int ref = (__double2hiint(acc->qunit) >> 20) & 0x7ff;
     for (long long pl = c0 + (long long)blockIdx.x * per + warp * GPW + gi; pl < c1;
          pl += (long long)gridDim.x * per) {
         const int p = (int)pl;
@@ -187,29 +224,50 @@ k_spread_fx(const int4* __restrict__ fac, const int2* __restrict__ xq,
         const int2* fx = xq + (size_t)(p - c0) * P;
         const int2 z = *reinterpret_cast<const int2*>(fy + P + k);
         unsigned long long* g0 = g64 + ((size_t)cell.x * Mp + cell.y) * Mp + cell.z + k;
+        int shift = 0;
+        if (!words) {
+            split_exponent(sorted[4 * (size_t)p + 3], &shift);
+            shift -= ref + 60;
+        }
 #pragma unroll 1
         for (int bc = 0; bc < P; bc += BC) {
             int yzh[BC], yzl[BC];
 #pragma unroll
             for (int b = 0; b < BC; ++b) {
                 const int2 y = __ldg(reinterpret_cast<const int2*>(fy + bc + b));
-                const long long cr = mad_wide(y.x, z.y, mad_wide(y.y, z.x, 0LL));
+                const long long cr = mad_wide(y.x, z.y, mad_wide(y.y, z.x, 1LL << 29));
                 const long long v = mad_wide(y.x, z.x, cr >> 30);
                 yzh[b] = (int)((v + (1 << 29)) >> 30);
                 yzl[b] = (int)v - (int)((unsigned)yzh[b] << 30);
             }
             unsigned long long* ga = g0 + (size_t)bc * Mp;
+            // start: what makes the cuts of the sum round without a preferred sign
+            // (errors of one sign add up over the weights of a cluster)
+            auto planes = [&](long long start, auto add) {
 #pragma unroll 1
-            for (int a = 0; a < P; ++a, ga += (size_t)Mp * Mp) {
-                const int2 x = __ldg(fx + a);
-                unsigned long long* g = ga;
+                for (int a = 0; a < P; ++a, ga += (size_t)Mp * Mp) {
+                    const int2 x = __ldg(fx + a);
+                    unsigned long long* g = ga;
 #pragma unroll
-                for (int b = 0; b < BC; ++b, g += Mp) {
-                    // + 4: the cut of three bits rounds
-                    const long long cr = mad_wide(x.x, yzl[b], mad_wide(x.y, yzh[b], 4LL << 30));
-                    const long long w = mad_wide(x.x, yzh[b], (long long)(int)(cr >> 30));
-                    atomicAdd(g, (unsigned long long)(w >> 3));
+                    for (int b = 0; b < BC; ++b, g += Mp) {
+                        const long long cr = mad_wide(x.x, yzl[b], mad_wide(x.y, yzh[b], start));
+                        add(g, mad_wide(x.x, yzh[b], (long long)(int)(cr >> 30)));
+                    }
                 }
+            };
+            if (words) {
+                // W cut, plus 4, cut by three bits: mean error (-1/2 + 1/2) / 8
+                planes(4LL << 30, [](unsigned long long* g, long long w) {
+                    atomicAdd(g, (unsigned long long)(w >> 3));
+                });
+            } else {
+                planes(1LL << 29, [shift](unsigned long long* g, long long w) {
+                    const double v = __ll2double_rn(w);
+                    const int hi = __double2hiint(v);
+                    if (((hi >> 20) & 0x7ff) + shift > 0)   // not for w = 0: shift <= -60
+                        atomicAdd(reinterpret_cast<double*>(g),
+                                  __hiloint2double(hi + (int)((unsigned)shift << 20), __double2loint(v)));
+                });
             }
         }
     }

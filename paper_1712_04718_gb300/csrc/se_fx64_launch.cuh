@@ -22,7 +22,8 @@ cudaError_t fx_spread_P(const FxParams& fp, const FxBufs& b, int c0, int c1, cud
     const int per = (kFxThreads / 32) * kFxGPW<P>;
     const int blocks = std::max(1, std::min((c1 - c0 + per - 1) / per, 1 << 20));
     k_spread_fx<P><<<blocks, kFxThreads, 0, s>>>((const int4*)b.fac, (const int2*)b.xq, b.cells,
-                                                 (unsigned long long*)b.g64, fp.kp.M + P - 1, c0, c1);
+                                                 (const double*)b.sorted, (unsigned long long*)b.g64,
+                                                 fp, b.acc, c0, c1);
     return cudaGetLastError();
 }
 

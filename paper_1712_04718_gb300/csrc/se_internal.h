@@ -47,6 +47,8 @@ struct Acc {
     double qscale, qunit;    // 1 / max|q| (a little less) and its inverse (k_bin)
     int tile_max;            // particles of the fullest tile (k_bin)
     unsigned int overflow;   // the transformed grid has Inf or NaN values (k_grid_split)
+    float qmean;             // mean |q| / max |q| (k_bin)
+    int pad;
 };
 
 // launchers (se_kernels_*.cu)

@@ -370,6 +370,7 @@ k_bin(const T* __restrict__ xyz, const T* __restrict__ q, const KParams<T> kp,
             const double qmax = __longlong_as_double((long long)sqm);
             acc->qscale = qmax > 0x1p-1000 ? (1.0 - 0x1p-50) / qmax : 0x1p+1000;
             acc->qunit = 1.0 / acc->qscale;
+            acc->qmean = (float)(t.y * acc->qscale) / (float)kp.N;
             *ticket = 0u;
         }
     }

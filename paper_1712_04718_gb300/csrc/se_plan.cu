@@ -192,6 +192,52 @@ size_t tsize(int prec) { return prec == SE_FP64 ? sizeof(double) : sizeof(float)
 size_t ik_gstride(const se_plan* p) { return ((size_t)p->M * p->M * p->M + 63) & ~(size_t)63; }
 size_t ik_cstride(const se_plan* p) { return ((size_t)p->M * p->M * (p->M / 2 + 1) + 31) & ~(size_t)31; }
 
+// What a grid point receives at most, in units of the weight of the largest
+// charge, if every tile holds one particle: the particles of a tile at distance
+// d (grid units, per dimension) weigh at most e^{-beta d^2}, so it is the cube of
+// the largest sum over the tiles of one dimension.  Two tiles meet at a face
+// point and the others are an edge or more away, except where the last tile is
+// narrow (M mod edge cells wide): there three lie within its width.
+double tile_crowd(const se_plan* p) {
+    const double beta = p->alpha * p->h * p->h;
+    double most = 0.0;
+    for (int x = 0; x < p->M; ++x) {
+        double sum = 0.0;
+        for (int a = 0; a < p->M; a += p->tile) {
+            const int b = std::min(a + p->tile, p->M);
+            const int d = x < a ? std::min(a - x, x + p->M - b)
+                                : (x > b ? std::min(x - b, a + p->M - x) : 0);
+            if (2 * d <= p->P + 2) sum += exp(-beta * d * d);   // farther ones do not reach
+        }
+        most = std::max(most, sum);
+    }
+    return most * most * most * (1.0 + 1e-6);
+}
+
+// Tile edge of the double-precision spread.  Its tiles only order the particles,
+// but their counts bound the sums of the integer grid (tile_crowd): eight tiles of
+// 32 particles of water just leave it kFxMinBits.  So edge 8 up to a mean count
+// of 16, and else, of the edges 4 to 8 with at most 20^3 tiles (the binning's scan
+// keeps 8192 counts in shared memory), the one with the lowest bound for a uniform
+// system.  Edge 4 for every system costs 5 us where the tiles outnumber the
+// particles (1000 charges, M = 64: the scan).
+int fx_tile(se_plan* p) {
+    const int n8 = (p->M + 7) / 8;
+    int best = 8;
+    double least = 0.0;
+    if (p->N <= (int64_t)16 * n8 * n8 * n8) return best;
+    for (int t = 8; t >= 4; --t) {
+        if (20 * t < p->M && t < 8) break;
+        p->tile = std::min(t, p->M);
+        const double b = tile_crowd(p) * t * t * t;
+        if (t == 8 || b < least) {
+            least = b;
+            best = t;
+        }
+    }
+    return best;
+}
+
 // Sec. 3 and Eq. 4.2: h = L/M, w = P h / 2, m = c sqrt(pi P),
 // eta = (2 w xi / m)^2, alpha = 2 xi^2 / eta, c_g = (2 xi^2 / (pi eta))^{3/2}.
 void derive(se_plan* p) {
@@ -202,7 +248,7 @@ void derive(se_plan* p) {
     p->alpha = 2.0 * p->xi * p->xi / p->eta;
     p->cg = pow(2.0 * p->xi * p->xi / (kPi * p->eta), 1.5);
     // spreading variant and tile edge
-    int tile = p->tune_tile > 0 ? p->tune_tile : 8;
+    int tile = p->tune_tile > 0 ? p->tune_tile : (p->prec == SE_FP64 ? fx_tile(p) : 8);
     if (p->P <= 16 && tile > 16) tile = 16;   // the staged regions' row stride allows 16
     if (tile > p->M) tile = p->M;
     p->tile = tile;
@@ -329,28 +375,6 @@ std::vector<double> green_table(const se_plan* p) {
         }
     }
     return g;
-}
-
-// What a grid point receives at most, in units of the weight of the largest
-// charge, if every tile holds one particle: the particles of a tile at distance
-// d (grid units, per dimension) weigh at most e^{-beta d^2}, so it is the cube of
-// the largest sum over the tiles of one dimension.  Two tiles meet at a face
-// point and the others are an edge or more away, except where the last tile is
-// narrow (M mod edge cells wide): there three lie within its width.
-double tile_crowd(const se_plan* p) {
-    const double beta = p->alpha * p->h * p->h;
-    double most = 0.0;
-    for (int x = 0; x < p->M; ++x) {
-        double sum = 0.0;
-        for (int a = 0; a < p->M; a += p->tile) {
-            const int b = std::min(a + p->tile, p->M);
-            const int d = x < a ? std::min(a - x, x + p->M - b)
-                                : (x > b ? std::min(x - b, a + p->M - x) : 0);
-            if (2 * d <= p->P + 2) sum += exp(-beta * d * d);   // farther ones do not reach
-        }
-        most = std::max(most, sum);
-    }
-    return most * most * most * (1.0 + 1e-6);
 }
 
 int prepare(se_plan* p) {

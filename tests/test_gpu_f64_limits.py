@@ -96,3 +96,35 @@ def test_charges_near_the_ends_of_the_range(scale):
     r = oracle.se_kspace(x, q, L, xi, M, P, cell_mode=64, grids=True)
     assert_close(H / scale, r["H"], TOL, label="spread grid")
     assert_close(phi / scale, r["phi"], 5 * TOL, label="phi")
+
+
+@pytest.mark.parametrize("n,P", [(20000, 8), (20000, 16)])
+def test_many_charges_of_both_signs_in_one_place(n, P):
+    """20 000 unit charges of alternating sign in eight cells.  The potential is
+    what their weights' cancellation leaves: rounding each weight to 2^-53 of
+    itself leaves sqrt(n sum w^2) 2^-53 of net charge, below 1e-13 of the
+    potential here; rounding it to 2^-45 of the largest weight, 1e-12."""
+    L, M = 2.0, 24
+    rng = np.random.default_rng(1)
+    x = np.vstack([0.31 + 2 * L / M * rng.random((n, 3)), L * rng.random((200, 3))])
+    q = np.where(np.arange(n + 200) % 2 == 0, 1.0, -1.0)
+    xi = _xi(L, M, P)
+    H, F, phi, E = _evaluate(x, q, L, xi, M, P)
+    r = oracle.se_kspace(x, q, L, xi, M, P, cell_mode=64, grids=True)
+    assert np.linalg.norm(phi - r["phi"]) < 1e-13 * np.linalg.norm(r["phi"])
+    assert np.linalg.norm(F - r["F"]) < 1e-13 * np.linalg.norm(r["F"])
+    assert abs(E - r["E"]) < 1e-13 * abs(r["E"])
+
+
+@pytest.mark.parametrize("big", [1.0, 30.0, 1e4, 1e8, 1e15])
+@pytest.mark.parametrize("P", [4, 8, 24])
+def test_grid_of_small_charges_beside_a_large_one(big, P):
+    """Grid points that only the small charges reach keep their digits."""
+    L, M = 2.0, 64
+    rng = np.random.default_rng(3)
+    x = np.vstack([[[0.05 * L] * 3], L * (0.45 + 0.2 * rng.random((400, 3)))])
+    q = np.concatenate([[big], rng.uniform(-1, 1, 400)])
+    H, _, _, _ = _evaluate(x, q, L, _xi(L, M, P), M, P)
+    r = oracle.se_kspace(x, q, L, _xi(L, M, P), M, P, cell_mode=64, grids=True)["H"]
+    s = slice(M // 3, 5 * M // 6)    # beyond the large charge's support
+    assert_close(H[s, s, s], r[s, s, s], TOL, label="spread grid")
