@@ -8,7 +8,7 @@ namespace se {
 
 #define SE_FX_EXTERN(P)                                                                           \
     extern template cudaError_t fx_scatter_P<P>(const double*, const double*, const FxParams&,    \
-                                                const FxBufs&, int, int, cudaStream_t);           \
+                                                const FxBufs&, int, int, bool, cudaStream_t);     \
     extern template cudaError_t fx_spread_P<P>(const FxParams&, const FxBufs&, int, int,          \
                                                cudaStream_t);                                     \
     extern template cudaError_t fx_gather_P<P>(const FxParams&, const FxBufs&, double*, double*,  \
@@ -110,9 +110,9 @@ k_grid_split(const double* __restrict__ grid, int M, int Mp, int p0, double gbou
 }
 
 cudaError_t scatter(const double* xyz, const double* q, const FxParams& fp, const FxBufs& b, int c0,
-                    int c1, cudaStream_t s) {
+                    int c1, bool again, cudaStream_t s) {
     switch (fp.kp.P) {
-#define SE_CASE(PP) case PP: return fx_scatter_P<PP>(xyz, q, fp, b, c0, c1, s);
+#define SE_CASE(PP) case PP: return fx_scatter_P<PP>(xyz, q, fp, b, c0, c1, again, s);
         SE_FOR_EACH_P(SE_CASE)
 #undef SE_CASE
         default: return cudaErrorInvalidValue;
@@ -127,7 +127,7 @@ cudaError_t fx_spread(const double* xyz, const double* q, const FxParams& fp, co
     cudaError_t e = cudaSuccess;
     for (int c0 = 0; c0 < N && e == cudaSuccess; c0 += b.cap) {
         const int c1 = (int)std::min<long long>(N, (long long)c0 + b.cap);
-        e = scatter(xyz, q, fp, b, c0, c1, s);
+        e = scatter(xyz, q, fp, b, c0, c1, c0 > 0, s);
         if (e != cudaSuccess) break;
         if (c0 == 0) mark(ctx, 1);
         if (only) return cudaSuccess;
@@ -147,9 +147,8 @@ cudaError_t fx_spread(const double* xyz, const double* q, const FxParams& fp, co
     return cudaGetLastError();
 }
 
-cudaError_t fx_gather(const double* xyz, const double* q, const FxParams& fp, const FxBufs& b,
-                      const double* grid, double* phi, double* F, double e_scale, double* E_out,
-                      const double* adj, cudaStream_t s) {
+cudaError_t fx_gather(const FxParams& fp, const FxBufs& b, const double* grid, double* phi,
+                      double* F, double e_scale, double* E_out, const double* adj, cudaStream_t s) {
     const int N = fp.kp.N;
     const int Mp = fp.kp.M + fp.kp.P - 1;
     const int blocks = (int)std::min(((long long)Mp * Mp + 7) / 8, 8LL * 152);
@@ -158,7 +157,7 @@ cudaError_t fx_gather(const double* xyz, const double* q, const FxParams& fp, co
     cudaError_t e = cudaGetLastError();
     for (int c0 = 0; e == cudaSuccess; c0 += b.cap) {
         const int c1 = (int)std::min<long long>(N, (long long)c0 + b.cap);
-        if (N > b.cap) e = scatter(xyz, q, fp, b, c0, c1, s);   // the factors of this range again
+        if (N > b.cap) e = scatter(nullptr, nullptr, fp, b, c0, c1, true, s);   // its factors again
         if (e != cudaSuccess) break;
         switch (fp.kp.P) {
 #define SE_CASE(PP) \

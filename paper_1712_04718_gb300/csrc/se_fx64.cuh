@@ -118,31 +118,44 @@ __device__ __forceinline__ double split_exponent(double q, int* field) {
 // for all a), so that dg costs integer operations only.
 // Bound by the FP64 pipe: two exponentials, a reciprocal and two operations a
 // factor.
+// again: the factors of a further range, or of a range once more, from the sorted
+// copies (the caller's arrays are read by the first scatter of a spread only).
 template <int P>
 __global__ void __launch_bounds__(64)
 k_scatter_fx(const double* __restrict__ xyz, const double* __restrict__ q, const FxParams fp,
              const int* __restrict__ slot, const int* __restrict__ tile_of,
              const int* __restrict__ tile_start, double* __restrict__ sorted,
              int* __restrict__ perm, int* __restrict__ cells, int4* __restrict__ fac,
-             int2* __restrict__ xq, const Acc* __restrict__ acc, int c0, int c1) {
+             int2* __restrict__ xq, const Acc* __restrict__ acc, int c0, int c1, bool again) {
     const KParams<double>& kp = fp.kp;
     __shared__ double sE3[P];   // exp(-beta a_c^2) 2^30
     if (threadIdx.x < P) sE3[threadIdx.x] = kp.E3[threadIdx.x] * 1073741824.0;
     __syncthreads();
     const int d = blockIdx.y;
     const int cut = 26 + fp.sd;   // 26 to 30
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < kp.N; i += gridDim.x * blockDim.x) {
-        const int dst = tile_start[tile_of[i]] + slot[i];
-        const double x = wrap_coord(xyz[3 * (size_t)i + d], kp.L, kp.invL);
-        double s;
-        const int c = cell_of(x, kp.invh, kp.M, &s);
-        sorted[4 * (size_t)dst + d] = x;
-        cells[4 * (size_t)dst + d] = c;
-        double qp = 0.0;
+    const int end = again ? c1 : kp.N;
+    for (int i = (again ? c0 : 0) + blockIdx.x * blockDim.x + threadIdx.x; i < end;
+         i += gridDim.x * blockDim.x) {
+        int dst = i, c;
+        double x, qp = 0.0;
+        if (again) {   // uniform
+            x = sorted[4 * (size_t)dst + d];
+            c = cells[4 * (size_t)dst + d];
+            if (d == 0) qp = sorted[4 * (size_t)dst + 3];
+        } else {
+            dst = tile_start[tile_of[i]] + slot[i];
+            x = wrap_coord(xyz[3 * (size_t)i + d], kp.L, kp.invL);
+            double s;
+            c = cell_of(x, kp.invh, kp.M, &s);
+            sorted[4 * (size_t)dst + d] = x;
+            cells[4 * (size_t)dst + d] = c;
+            if (d == 0) {
+                qp = q[i];
+                sorted[4 * (size_t)dst + 3] = qp;
+                perm[dst] = i;
+            }
+        }
         if (d == 0) {
-            qp = q[i];
-            sorted[4 * (size_t)dst + 3] = qp;
-            perm[dst] = i;
             const int bits = grid_bits(acc, fp);
             int field;
             if (bits > 0) qp *= acc->qscale * pow2i(bits - 57);

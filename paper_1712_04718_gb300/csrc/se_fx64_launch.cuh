@@ -9,11 +9,12 @@ namespace se {
 
 template <int P>
 cudaError_t fx_scatter_P(const double* xyz, const double* q, const FxParams& fp, const FxBufs& b,
-                         int c0, int c1, cudaStream_t s) {
-    const int blocks = std::max(1, std::min((fp.kp.N + 63) / 64, 1 << 18));
+                         int c0, int c1, bool again, cudaStream_t s) {
+    const long long n = again ? c1 - c0 : fp.kp.N;
+    const int blocks = (int)std::max(1LL, std::min((n + 63) / 64, 1LL << 18));
     k_scatter_fx<P><<<dim3(blocks, 3), 64, 0, s>>>(xyz, q, fp, b.slot, b.tile_of, b.tile_start,
                                            (double*)b.sorted, b.perm, b.cells, (int4*)b.fac,
-                                           (int2*)b.xq, b.acc, c0, c1);
+                                           (int2*)b.xq, b.acc, c0, c1, again);
     return cudaGetLastError();
 }
 
@@ -41,7 +42,7 @@ cudaError_t fx_gather_P(const FxParams& fp, const FxBufs& b, double* phi, double
 
 #define SE_FX_INSTANTIATE(P)                                                                      \
     template cudaError_t fx_scatter_P<P>(const double*, const double*, const FxParams&,           \
-                                         const FxBufs&, int, int, cudaStream_t);                  \
+                                         const FxBufs&, int, int, bool, cudaStream_t);            \
     template cudaError_t fx_spread_P<P>(const FxParams&, const FxBufs&, int, int, cudaStream_t);  \
     template cudaError_t fx_gather_P<P>(const FxParams&, const FxBufs&, double*, double*, double, \
                                         double*, const double*, int, int, cudaStream_t);

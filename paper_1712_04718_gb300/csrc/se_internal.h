@@ -124,9 +124,8 @@ struct FxBufs {
 // (with `only` the particles in tile order and the factors, no spread)
 cudaError_t fx_spread(const double* xyz, const double* q, const FxParams& fp, const FxBufs& b,
                       bool only, cudaStream_t s, void (*mark)(void*, int), void* ctx);
-cudaError_t fx_gather(const double* xyz, const double* q, const FxParams& fp, const FxBufs& b,
-                      const double* grid, double* phi, double* F, double e_scale, double* E_out,
-                      const double* adj, cudaStream_t s);
+cudaError_t fx_gather(const FxParams& fp, const FxBufs& b, const double* grid, double* phi,
+                      double* F, double e_scale, double* E_out, const double* adj, cudaStream_t s);
 
 // Kernel parameters for an FP64 evaluation without a plan (se_plan.cu).
 int make_kparams_f64(int64_t N, double L, double xi, int M, int P, int tile, KParams<double>* out);

@@ -747,8 +747,7 @@ int do_scale(se_plan* p, double* E_grid) {
 }
 
 template <typename T>
-int do_gather(se_plan* p, const void* xyz, const void* q, void* phi, void* F, double* E,
-              const double* adj = nullptr) {
+int do_gather(se_plan* p, void* phi, void* F, double* E, const double* adj = nullptr) {
     const KParams<T> kp = make_kparams<T>(p);
     using V = se::v4_t<T>;
     // ik forces: potential and force from the four grids with the plain window;
@@ -761,8 +760,8 @@ int do_gather(se_plan* p, const void* xyz, const void* q, void* phi, void* F, do
                                            p->partials + 4 * se::kMaxPartials, p->tickets + 2,
                                            p->acc, 0.5, E, false, p->stream));
     else if constexpr (std::is_same<T, double>::value)
-        SE_CUDA(se::fx_gather((const T*)xyz, (const T*)q, fx_params(p), fx_bufs(p),
-                              (const T*)p->grid_gather, (T*)phi, (T*)F, 0.5, E, adj, p->stream));
+        SE_CUDA(se::fx_gather(fx_params(p), fx_bufs(p), (const T*)p->grid_gather, (T*)phi, (T*)F, 0.5, E,
+                              adj, p->stream));
     else
         SE_CUDA(se::launch_gather<T>((const V*)p->sorted, p->perm, (const T*)p->grid_gather, (T*)phi,
                                      (T*)F, kp, p->partials + 4 * se::kMaxPartials, p->tickets + 2,
@@ -798,11 +797,11 @@ int evaluate(se_plan* p, const void* xyz, const void* q, void* F, void* phi, dou
     if (p->prec == SE_FP64) {
         SE_TRY(do_spread<double>(p, xyz, q));
         SE_TRY(do_scale<double>(p, energy_only ? dE : nullptr));
-        if (!energy_only) SE_TRY(do_gather<double>(p, xyz, q, phi, F, dE));
+        if (!energy_only) SE_TRY(do_gather<double>(p, phi, F, dE));
     } else {
         SE_TRY(do_spread<float>(p, xyz, q));
         SE_TRY(do_scale<float>(p, energy_only ? dE : nullptr));
-        if (!energy_only) SE_TRY(do_gather<float>(p, xyz, q, phi, F, dE));
+        if (!energy_only) SE_TRY(do_gather<float>(p, phi, F, dE));
     }
     return SE_OK;
 }
@@ -1126,8 +1125,7 @@ int se_gather(se_plan* p, const void* xyz, const void* q, void* phi, void* F, do
     if (!p || (p->N > 0 && (!xyz || !q))) return SE_ERR_ARG;
     if (!p->ready || !p->have_scale) return SE_ERR_ARG;
     if (p->variant >= 3) return fast_gather(p, phi, F, E);
-    return p->prec == SE_FP64 ? do_gather<double>(p, xyz, q, phi, F, E)
-                              : do_gather<float>(p, xyz, q, phi, F, E);
+    return p->prec == SE_FP64 ? do_gather<double>(p, phi, F, E) : do_gather<float>(p, phi, F, E);
 }
 
 int se_adjoint(se_plan* p, const void* xyz, const void* q, const double* gE, void* grad_x,
@@ -1135,8 +1133,8 @@ int se_adjoint(se_plan* p, const void* xyz, const void* q, const double* gE, voi
     if (!p || !gE || (p->N > 0 && (!xyz || !q))) return SE_ERR_ARG;
     if (!p->ready || !p->have_scale) return SE_ERR_ARG;
     if (p->variant >= 3) return fast_gather(p, grad_q, grad_x, nullptr, gE);
-    return p->prec == SE_FP64 ? do_gather<double>(p, xyz, q, grad_q, grad_x, nullptr, gE)
-                              : do_gather<float>(p, xyz, q, grad_q, grad_x, nullptr, gE);
+    return p->prec == SE_FP64 ? do_gather<double>(p, grad_q, grad_x, nullptr, gE)
+                              : do_gather<float>(p, grad_q, grad_x, nullptr, gE);
 }
 
 int se_energy_force(se_plan* p, const void* xyz, const void* q, double* E, void* F, void* phi) {

@@ -164,3 +164,53 @@ def test_gather_errors_have_no_preferred_sign(P):
             ref *= ld(-2.0) * ld(p["alpha"]) * ld(p["h"]) ** 4 * ld(p["cg"]) * ld(q[i])
             err[i, d] = float((ld(F[i, d].item()) - ref) * ld(q[i]))
     assert (np.abs(err.mean(0)) < err.std(0)).all(), (err.mean(0), err.std(0))
+
+
+def test_ranges_gather_from_the_plans_copies():
+    """More particles than one range of window factors holds (4 GB at 1792
+    bytes a particle).  Results of a second range are those of any other
+    particle, and the gather needs the positions and charges of the spread no
+    more: writing the potential over the charges, or changing the positions
+    between the steps, changes nothing."""
+    L, M, P, N = 3.0, 40, 32, 2_500_000
+    g = torch.Generator(device="cuda").manual_seed(1)
+    x = L * torch.rand(N, 3, generator=g, device="cuda", dtype=torch.float64)
+    q = torch.where(torch.arange(N, device="cuda") % 2 == 0, 1.0, -1.0).double()
+    plan = se.Plan(N, L, _xi(L, M, P), M, P, precision="fp64")
+    F, phi = torch.empty_like(x), torch.empty_like(q)
+    plan.evaluate(x, q, F, phi)
+    # the same grid seen by particles of both ends of the tile order, as a
+    # system of test charges too small to change it
+    Ht = plan.copy_grid(1)
+    p = plan.params()
+    beta = p["alpha"] * p["h"] ** 2
+    s = torch.randperm(N, generator=torch.Generator().manual_seed(2))[:4000].cuda()
+    c = torch.floor(x[s] * (M / L)).long()
+    a = torch.arange(P, device="cuda")
+    dz = (a - (P - 1) / 2)[None, :, None] - (x[s] * (M / L) - c - 0.5)[:, None, :]
+    w = torch.exp(-beta * dz ** 2)
+    idx = (c[:, None, :] - P // 2 + 1 + a[None, :, None]) % M
+    ref, refF = torch.empty(4000, device="cuda").double(), torch.empty(4000, 3, device="cuda").double()
+    for k in range(0, 4000, 100):
+        i, v = idx[k:k + 100], w[k:k + 100]
+        V = Ht[i[:, :, None, None, 0], i[:, None, :, None, 1], i[:, None, None, :, 2]]
+        ref[k:k + 100] = torch.einsum("nabc,na,nb,nc->n", V, v[..., 0], v[..., 1], v[..., 2])
+        for d in range(3):
+            u = [v[..., e] * dz[k:k + 100, :, e] if e == d else v[..., e] for e in range(3)]
+            refF[k:k + 100, d] = torch.einsum("nabc,na,nb,nc->n", V, *u)
+    ref *= p["h"] ** 3 * p["cg"]
+    refF *= -2 * p["alpha"] * p["h"] ** 4 * p["cg"] * q[s][:, None]
+    assert_close(phi[s].cpu().numpy(), ref.cpu().numpy(), 5 * TOL, label="phi")
+    assert_close(F[s].cpu().numpy(), refF.cpu().numpy(), 5 * TOL, label="F", q=q[s].cpu().numpy())
+    q2, F2 = q.clone(), torch.empty_like(x)
+    plan.set_graph(False)
+    plan.evaluate(x, q2, F2, q2)      # phi over q
+    assert torch.equal(q2, phi) or float((q2 - phi).norm() / phi.norm()) < TOL
+    assert float((F2 - F).norm() / F.norm()) < TOL
+    plan.spread(x, q)
+    plan.scale()
+    x2 = x.clone().roll(1, 0)
+    plan.gather(x2, q, phi=q2, F=F2)
+    assert float((q2 - phi).norm() / phi.norm()) < TOL
+    assert float((F2 - F).norm() / F.norm()) < TOL
+    plan.close()
