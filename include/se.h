@@ -72,7 +72,10 @@ typedef struct se_plan se_plan;
  * N >= 0 (N = 0 gives zero results), L > 0, xi > 0, 2 <= P <= min(M, 32),
  * P even; otherwise SE_ERR_ARG (SE_ERR_UNSUPPORTED for odd P or P > 32).
  * Device memory is allocated on the current CUDA device at the first
- * computing call.  *out is set to NULL on failure. */
+ * computing call; beside grids, spectra, tables and sort buffers, SE_FP64 takes
+ * 8 (M + P - 1)^3 bytes for its integer grid and 56 P bytes a particle of window
+ * factors, at most 4 GB (more particles are taken in ranges; less where memory
+ * is short).  *out is set to NULL on failure. */
 int se_plan_create(se_plan **out, int64_t N, double L, double xi, int M, int P);
 
 /* Release every resource of the plan (NULL is accepted). */

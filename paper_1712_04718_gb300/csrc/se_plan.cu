@@ -91,7 +91,6 @@ struct se_plan {
     double fx_crowd = 0.0;               // tile_crowd
     cudaStream_t fft_stream = nullptr;   // stream the FFT plans were last given
     bool fft_stream_set = false;
-    void* fx_split = nullptr;
     void* fx_grid = nullptr;
     double* fx_parts = nullptr;
     int fx_nparts = 0;
@@ -297,7 +296,7 @@ void release_device(se_plan* p) {
                     p->tile_start, p->slot, p->tile_of, p->perm, p->sorted, p->partials,
                     p->tickets, p->acc, p->dE, p->h_xyz, p->h_q, p->h_F, p->h_phi, p->g64, p->tw, p->green_f,
                     p->bucket, p->bucket_idx, p->cgrid_ik, p->part, p->fx_fac, p->fx_xq,
-                    p->fx_cells, p->fx_top, p->fx_split, p->fx_grid, p->fx_parts};
+                    p->fx_cells, p->fx_top, p->fx_grid, p->fx_parts};
     for (void* b : bufs)
         if (b) cudaFree(b);
     p->grid_spread = p->grid_gather = p->cgrid = p->sorted = p->tw = p->bucket = nullptr;
@@ -307,7 +306,7 @@ void release_device(se_plan* p) {
     p->fx_fac = p->fx_xq = nullptr;
     p->fx_cells = nullptr;
     p->fx_top = nullptr;
-    p->fx_split = p->fx_grid = nullptr;
+    p->fx_grid = nullptr;
     p->fx_parts = nullptr;
     p->g64 = nullptr;
     p->green_f = nullptr;
@@ -377,6 +376,8 @@ std::vector<double> green_table(const se_plan* p) {
     return g;
 }
 
+bool fx_spread_used(const se_plan* p) { return p->prec == SE_FP64 && p->variant != 2; }
+
 int prepare(se_plan* p) {
     int dev = 0;
     SE_CUDA(cudaGetDevice(&dev));
@@ -405,7 +406,11 @@ int prepare(se_plan* p) {
     if (rc == SE_OK && fast) rc = dalloc((void**)&p->green_f, nc * sizeof(float));
     if (rc == SE_OK) rc = dalloc(&p->grid_gather, ik ? 4 * ik_gstride(p) * ts : M3 * ts);
     if (rc == SE_OK && ik) rc = dalloc(&p->cgrid_ik, 3 * ik_cstride(p) * 2 * ts);
-    if (rc == SE_OK) rc = dalloc(&p->cgrid, nc * 2 * ts);
+    // double precision: the gather's split grid (se_fx64.cuh) takes the place of
+    // the spectrum, which the inverse transform has consumed
+    const size_t Mp = (size_t)p->M + p->P - 1, Mp3 = Mp * Mp * Mp;
+    const size_t split = p->prec == SE_FP64 ? Mp3 * 2 * sizeof(int) : 0;
+    if (rc == SE_OK) rc = dalloc(&p->cgrid, std::max(nc * 2 * ts, split));
     if (rc == SE_OK) rc = dalloc((void**)&p->green, nc * sizeof(double));
     if (rc == SE_OK) rc = dalloc((void**)&p->tile_count, (size_t)p->ntiles * sizeof(int));
     if (rc == SE_OK) rc = dalloc((void**)&p->tile_start, ((size_t)p->ntiles + 1) * sizeof(int));
@@ -418,17 +423,13 @@ int prepare(se_plan* p) {
     if (rc == SE_OK) rc = dalloc((void**)&p->acc, sizeof(Acc));
     if (rc == SE_OK) rc = dalloc((void**)&p->dE, sizeof(double));
     if (p->prec == SE_FP64) {
-        const size_t per = (size_t)56 * p->P;   // bytes of factors a particle
-        p->fx_cap = (int)std::max<size_t>(1, std::min(N, se::kFxFactorBytes / per));
-        if (rc == SE_OK) rc = dalloc(&p->fx_fac, (size_t)p->fx_cap * 48 * p->P);
-        if (rc == SE_OK) rc = dalloc(&p->fx_xq, (size_t)p->fx_cap * 8 * p->P);
         if (rc == SE_OK) rc = dalloc((void**)&p->fx_cells, N * 4 * sizeof(int));
         if (rc == SE_OK) rc = dalloc((void**)&p->fx_top, sizeof(int));
-        const size_t Mp = (size_t)p->M + p->P - 1;
-        if (rc == SE_OK) rc = dalloc(&p->fx_split, Mp * Mp * Mp * 2 * sizeof(int));
-        if (rc == SE_OK) rc = dalloc(&p->fx_grid, Mp * Mp * Mp * sizeof(long long));
-        if (rc == SE_OK && cudaMemset(p->fx_grid, 0, Mp * Mp * Mp * sizeof(long long)) != cudaSuccess)
-            rc = SE_ERR_CUDA;
+        if (fx_spread_used(p)) {
+            if (rc == SE_OK) rc = dalloc(&p->fx_grid, Mp3 * sizeof(long long));
+            if (rc == SE_OK && cudaMemset(p->fx_grid, 0, Mp3 * sizeof(long long)) != cudaSuccess)
+                rc = SE_ERR_CUDA;
+        }
         p->fx_nparts = (int)std::min<size_t>(1 << 16, N + 1);
         if (rc == SE_OK) rc = dalloc((void**)&p->fx_parts, (size_t)p->fx_nparts * sizeof(double));
     }
@@ -496,6 +497,24 @@ int prepare(se_plan* p) {
         return SE_ERR_CUFFT;
     }
     p->have_fft = true;
+    if (p->prec == SE_FP64) {
+        // last, so that the window factors take what is left: where memory is
+        // short, of shorter ranges (down to 2^14 particles)
+        const size_t per = (size_t)56 * p->P;   // bytes of factors a particle
+        p->fx_cap = (int)std::max<size_t>(1, std::min(N, se::kFxFactorBytes / per));
+        for (;; p->fx_cap = (p->fx_cap + 1) / 2) {
+            rc = dalloc(&p->fx_fac, (size_t)p->fx_cap * 48 * p->P);
+            if (rc == SE_OK) rc = dalloc(&p->fx_xq, (size_t)p->fx_cap * 8 * p->P);
+            if (rc == SE_OK) break;
+            cudaGetLastError();
+            if (p->fx_fac) cudaFree(p->fx_fac);
+            p->fx_fac = nullptr;
+            if (p->fx_cap <= (1 << 14)) {
+                release_device(p);
+                return rc;
+            }
+        }
+    }
     p->spread_clean = true;
     p->have_spread = p->have_scale = false;
     p->ready = true;
@@ -513,7 +532,6 @@ void invalidate(se_plan* p) {
 // The grid that the spread adds to: the fixed-point one of the single-precision
 // pipeline, the padded integer one of the double-precision spread, or the real
 // one; and its values (all of 8 bytes but for float grids).
-bool fx_spread_used(const se_plan* p) { return p->prec == SE_FP64 && p->variant != 2; }
 void* spread_target(const se_plan* p, size_t* n) {
     const size_t e = (size_t)p->M + (fx_spread_used(p) ? p->P - 1 : 0);
     *n = e * e * e;
@@ -590,7 +608,7 @@ se::FxBufs fx_bufs(se_plan* p) {
     b.tile_start = p->tile_start;
     b.perm = p->perm;
     b.sorted = p->sorted;
-    b.split = p->fx_split;
+    b.split = p->cgrid;
     b.top = p->fx_top;
     b.parts = p->fx_parts;
     b.nparts = p->fx_nparts;

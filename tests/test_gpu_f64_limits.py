@@ -214,3 +214,28 @@ def test_ranges_gather_from_the_plans_copies():
     assert float((q2 - phi).norm() / phi.norm()) < TOL
     assert float((F2 - F).norm() / F.norm()) < TOL
     plan.close()
+
+
+def test_memory_of_a_plan():
+    """Only the integer spread has a padded integer grid, and the gather's copy
+    of the grid shares the spectrum's memory."""
+    M, N = 256, 10
+
+    def used(P, **kw):
+        plan = se.Plan(N, 3.0, 1.0, M, P, precision="fp64", **kw)
+        x = 3.0 * torch.rand(N, 3, device="cuda", dtype=torch.float64)
+        q = torch.rand(N, device="cuda", dtype=torch.float64) - 0.5
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        plan.spread(x, q)
+        torch.cuda.synchronize()
+        free -= torch.cuda.mem_get_info()[0]
+        plan.close()
+        return free
+
+    used(8)                    # loads the kernels
+    mb = 1 << 20
+    grid, pad = 8 * M ** 3, 8 * (M + 31) ** 3
+    direct = used(32, spread_variant=2)
+    assert abs(used(32, spread_variant=1) - direct - pad) < 8 * mb
+    assert direct - used(2, spread_variant=2) < pad - grid + 8 * mb
