@@ -2,4 +2,5 @@
 #include "se_launch.cuh"
 namespace se {
 SE_INSTANTIATE(double)
+SE_INSTANTIATE_GATHER(double)
 }

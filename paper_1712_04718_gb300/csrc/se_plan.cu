@@ -87,6 +87,7 @@ struct se_plan {
     int fx_cap = 0;
     int* fx_cells = nullptr;
     int* fx_top = nullptr;
+    bool fx = false;                     // the integer gather is used (derive)
     double fx_gbound = 0.0;
     double fx_crowd = 0.0;               // tile_crowd
     cudaStream_t fft_stream = nullptr;   // stream the FFT plans were last given
@@ -213,6 +214,20 @@ double tile_crowd(const se_plan* p) {
     return most * most * most * (1.0 + 1e-6);
 }
 
+// Double precision, few particles on a large grid: the integer spread and gather
+// pass over the padded grid three times (integer grid to FP64, its clearing, the
+// split), about 9 ps a point; the FP64 reductions of variant 2 and the FP64 gather
+// do not, but take 10 ps a support point more and 0.3 P^2 us for a particle's
+// chain of FP64 operations.  The line lies where the two are equal; on both sides
+// of it (integers / FP64): M = 256: 1000 charges, P = 8: 3943 / 3796 us; 10 000,
+// P = 8: 3973 / 3888; 300, P = 16: 3962 / 3863; M = 160: 3000, P = 8: 1246 / 1227;
+// 50, P = 16: 1256 / 1292; M = 128: 100, P = 4: 556 / 543; 300, P = 12: 574 / 628;
+// M = 96: 300, P = 4: 265 / 267; 50, P = 8: 269 / 283.
+bool few_particles(const se_plan* p) {
+    const double Mp = p->M + p->P - 1, P = p->P;
+    return Mp * Mp * Mp > P * P * P * p->N + 4e4 * P * P + 4e5;
+}
+
 // Tile edge of the double-precision spread.  Its tiles only order the particles,
 // but their counts bound the sums of the integer grid (tile_crowd): eight tiles of
 // 32 particles of water just leave it kFxMinBits.  So edge 8 up to a mean count
@@ -259,8 +274,9 @@ void derive(se_plan* p) {
     if (variant == 4 && (p->prec == SE_FP64 || p->M > se::kFastMaxM)) variant = 0;
     // ik forces need the three extra inverse transforms of the cuFFT pipeline
     if (p->force_mode == SE_FORCE_IK && variant >= 3) variant = 0;
+    p->fx = p->prec == SE_FP64 && (variant == 1 || !few_particles(p));
     if (variant == 0) {
-        if (p->prec == SE_FP64) variant = 1;
+        if (p->prec == SE_FP64) variant = p->fx ? 1 : 2;
         else variant = (fast_ok && p->force_mode != SE_FORCE_IK) ? 3 : 1;
     }
     if (p->prec == SE_FP32 && variant == 2) variant = 1;  // the compensated sum needs the tiles
@@ -376,7 +392,7 @@ std::vector<double> green_table(const se_plan* p) {
     return g;
 }
 
-bool fx_spread_used(const se_plan* p) { return p->prec == SE_FP64 && p->variant != 2; }
+bool fx_spread_used(const se_plan* p) { return p->fx && p->variant != 2; }
 
 int prepare(se_plan* p) {
     int dev = 0;
@@ -409,7 +425,7 @@ int prepare(se_plan* p) {
     // double precision: the gather's split grid (se_fx64.cuh) takes the place of
     // the spectrum, which the inverse transform has consumed
     const size_t Mp = (size_t)p->M + p->P - 1, Mp3 = Mp * Mp * Mp;
-    const size_t split = p->prec == SE_FP64 ? Mp3 * 2 * sizeof(int) : 0;
+    const size_t split = p->fx ? Mp3 * 2 * sizeof(int) : 0;
     if (rc == SE_OK) rc = dalloc(&p->cgrid, std::max(nc * 2 * ts, split));
     if (rc == SE_OK) rc = dalloc((void**)&p->green, nc * sizeof(double));
     if (rc == SE_OK) rc = dalloc((void**)&p->tile_count, (size_t)p->ntiles * sizeof(int));
@@ -422,7 +438,7 @@ int prepare(se_plan* p) {
     if (rc == SE_OK) rc = dalloc((void**)&p->tickets, 8 * sizeof(unsigned));
     if (rc == SE_OK) rc = dalloc((void**)&p->acc, sizeof(Acc));
     if (rc == SE_OK) rc = dalloc((void**)&p->dE, sizeof(double));
-    if (p->prec == SE_FP64) {
+    if (p->fx) {
         if (rc == SE_OK) rc = dalloc((void**)&p->fx_cells, N * 4 * sizeof(int));
         if (rc == SE_OK) rc = dalloc((void**)&p->fx_top, sizeof(int));
         if (fx_spread_used(p)) {
@@ -438,7 +454,7 @@ int prepare(se_plan* p) {
         return rc;
     }
     std::vector<double> g = green_table(p);
-    if (p->prec == SE_FP64) {
+    if (p->fx) {
         p->fx_crowd = tile_crowd(p);
         // sum of G over the whole spectrum: the half spectrum's inner planes twice
         double sum = 0.0;
@@ -497,7 +513,7 @@ int prepare(se_plan* p) {
         return SE_ERR_CUFFT;
     }
     p->have_fft = true;
-    if (p->prec == SE_FP64) {
+    if (p->fx) {
         // last, so that the window factors take what is left: where memory is
         // short, of shorter ranges (down to 2^14 particles)
         const size_t per = (size_t)56 * p->P;   // bytes of factors a particle
@@ -693,25 +709,24 @@ int do_spread(se_plan* p, const void* xyz, const void* q) {
     SE_CUDA(se::launch_bin<T>((const T*)xyz, (const T*)q, kp, p->tile_count, p->slot, p->tile_of,
                               p->tile_start, p->partials, p->tickets + 0, p->acc, p->stream));
     timing_mark(p, 0);
+    bool done = false;
     if constexpr (std::is_same<T, double>::value) {
-        // factors (for the gather too), then the spread; variant 2 spreads with
-        // global FP64 reductions instead
-        SE_CUDA(se::fx_spread((const double*)xyz, (const double*)q, fx_params(p), fx_bufs(p),
-                              p->variant == 2, p->stream, mark_cb, p));
-        if (p->N > 0 && p->variant == 2)
-            SE_CUDA(se::launch_spread_direct<T>((const V*)p->sorted, (T*)p->grid_spread, kp, p->stream));
-    } else {
+        // factors (for the gather too), then the spread
+        if (p->fx)
+            SE_CUDA(se::fx_spread((const double*)xyz, (const double*)q, fx_params(p), fx_bufs(p),
+                                  p->variant == 2, p->stream, mark_cb, p));
+        done = p->fx;
+    }
+    if (!done) {
         SE_CUDA(se::launch_scatter<T>((const T*)xyz, (const T*)q, kp, p->slot, p->tile_of,
                                       p->tile_start, (V*)p->sorted, p->perm, p->stream));
         timing_mark(p, 1);
-        if (p->N > 0) {
-            if (p->variant == 2)
-                SE_CUDA(se::launch_spread_direct<T>((const V*)p->sorted, (T*)p->grid_spread, kp, p->stream));
-            else
-                SE_CUDA(se::launch_spread_tiled<T>((const V*)p->sorted, p->tile_start, (T*)p->grid_spread,
-                                                   kp, p->prec == SE_FP32, p->acc, p->stream));
-        }
     }
+    if (p->N > 0 && p->variant == 2)
+        SE_CUDA(se::launch_spread_direct<T>((const V*)p->sorted, (T*)p->grid_spread, kp, p->stream));
+    else if (p->N > 0 && p->prec != SE_FP64)
+        SE_CUDA(se::launch_spread_tiled<T>((const V*)p->sorted, p->tile_start, (T*)p->grid_spread,
+                                           kp, p->prec == SE_FP32, p->acc, p->stream));
     timing_mark(p, 2);
     p->spread_clean = false;
     p->have_spread = true;
@@ -777,10 +792,11 @@ int do_gather(se_plan* p, void* phi, void* F, double* E, const double* adj = nul
                                            ik_gstride(p), (T*)phi, (T*)F, kp,
                                            p->partials + 4 * se::kMaxPartials, p->tickets + 2,
                                            p->acc, 0.5, E, false, p->stream));
-    else if constexpr (std::is_same<T, double>::value)
-        SE_CUDA(se::fx_gather(fx_params(p), fx_bufs(p), (const T*)p->grid_gather, (T*)phi, (T*)F, 0.5, E,
-                              adj, p->stream));
-    else
+    else if (p->fx) {
+        if constexpr (std::is_same<T, double>::value)
+            SE_CUDA(se::fx_gather(fx_params(p), fx_bufs(p), (const T*)p->grid_gather, (T*)phi, (T*)F,
+                                  0.5, E, adj, p->stream));
+    } else
         SE_CUDA(se::launch_gather<T>((const V*)p->sorted, p->perm, (const T*)p->grid_gather, (T*)phi,
                                      (T*)F, kp, p->partials + 4 * se::kMaxPartials, p->tickets + 2,
                                      p->acc, 0.5, E, adj, p->stream));

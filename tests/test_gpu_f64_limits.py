@@ -239,3 +239,36 @@ def test_memory_of_a_plan():
     direct = used(32, spread_variant=2)
     assert abs(used(32, spread_variant=1) - direct - pad) < 8 * mb
     assert direct - used(2, spread_variant=2) < pad - grid + 8 * mb
+
+
+@pytest.mark.parametrize("N,M,P,few", [(0, 128, 4, True), (2, 129, 2, True), (100, 128, 4, True),
+                                       (700, 160, 8, True), (700, 128, 8, False),
+                                       (10, 33, 16, False)])
+def test_few_particles_on_a_large_grid(N, M, P, few):
+    """The FP64 path that few particles take gives what the integer one (variant
+    1) gives, in every mode of evaluation."""
+    L = 2.0
+    x, q = systems.uniform_charges(max(N, 1), L, seed=N + M)
+    xd, qd = _dev(x[:N].reshape(N, 3)), _dev(q[:N])
+    one = torch.ones(1, dtype=torch.float64, device="cuda")
+    out = {}
+    for variant in (0, 1):
+        plan = se.Plan(N, L, _xi(L, M, P), M, P, precision="fp64", spread_variant=variant)
+        assert plan.params()["spread_variant"] == (2 if few and variant == 0 else 1)
+        r = []
+        for mode in ("analytic", "ik"):
+            plan.set_force_mode(mode)
+            F, phi, E = torch.empty_like(xd), torch.empty_like(qd), torch.zeros_like(one)
+            plan.evaluate(xd, qd, F, phi, E)
+            phi1, E0 = torch.empty_like(qd), torch.zeros_like(one)
+            plan.evaluate(xd, qd, None, phi1, None)
+            plan.evaluate(xd, qd, None, None, E0)
+            gx, gq = torch.empty_like(xd), torch.empty_like(qd)
+            plan.adjoint(xd, qd, one, gx, gq)
+            r += [F, phi, E, phi1, E0, gx, gq, plan.copy_grid(1)]
+            plan.spread(xd, qd)
+            r.append(plan.copy_grid(0))
+        out[variant] = [t.cpu().numpy() for t in r]
+        plan.close()
+    for a, b in zip(out[0], out[1]):
+        assert np.linalg.norm(a - b) <= 5 * TOL * np.linalg.norm(b)
