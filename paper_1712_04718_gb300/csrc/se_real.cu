@@ -493,19 +493,23 @@ struct PairScales {
 };
 
 constexpr int kPair64Warps = 6;
-constexpr int kCap64 = 2048;        // staged candidates (96 KB: two CTAs per SM)
+// Staged candidates: at most 2048 (96 KB: two CTAs per SM); half a box's mean count
+// over, and at least 512 (24 KB: five CTAs, as many as the registers allow), where
+// fewer will do (rs_run): sparse cells are many short CTAs (20 000 particles in
+// 40^3 cells: 780 us at 2048, 548 at 512; with FP64 arithmetic for every pair 755).
+constexpr int kCap64 = 2048, kCap64Min = 512;
 constexpr int kTest64 = 128;        // candidates tested per step
 constexpr int kQueue64 = kTest64 + 32;
 
 __global__ void __launch_bounds__(32 * kPair64Warps)
 k_rs_pairs64(const se::d4* __restrict__ sorted, const se::f4* __restrict__ sorted_f,
-             const int* __restrict__ start, const int* __restrict__ perm, int nc, int K, double L,
-             double rc2, float rc2_f, const PairScales sc, double kc, const double2* __restrict__ table,
+             const int* __restrict__ start, const int* __restrict__ perm, int cap, int nc, int K,
+             double L, double rc2, float rc2_f, const PairScales sc, double kc, const double2* __restrict__ table,
              double* __restrict__ phi, double* __restrict__ F, int accumulate,
              double* __restrict__ partials, unsigned* ticket, double* E_out) {
     extern __shared__ __align__(32) unsigned char smem_raw[];
     se::d4* nb = reinterpret_cast<se::d4*>(smem_raw);
-    se::f4* nf = reinterpret_cast<se::f4*>(smem_raw + kCap64 * sizeof(se::d4));
+    se::f4* nf = reinterpret_cast<se::f4*>(smem_raw + cap * sizeof(se::d4));
     __shared__ int s_b0[kMaxStencil], s_off[kMaxStencil + 1];
     __shared__ unsigned char s_sh[kMaxStencil];
     __shared__ unsigned short s_q[kPair64Warps][kQueue64];
@@ -563,9 +567,9 @@ k_rs_pairs64(const se::d4* __restrict__ sorted, const se::f4* __restrict__ sorte
             fy += fq * dy;
             fz += fq * dz;
         };
-        for (int c0 = 0; c0 < total; c0 += kCap64) {
-            const int filled = min(kCap64, total - c0);
-            if (pass0 == 0 || total > kCap64) {   // one chunk: staged once for all passes
+        for (int c0 = 0; c0 < total; c0 += cap) {
+            const int filled = min(cap, total - c0);
+            if (pass0 == 0 || total > cap) {   // one chunk: staged once for all passes
                 __syncthreads();
                 for (int t = threadIdx.x; t < filled; t += blockDim.x) {
                     const int k = stencil_cell(s_off, W3, c0 + t);
@@ -797,12 +801,16 @@ int rs_run(se_real* r, const void* xyz, const void* q, void* F, void* phi, doubl
         const bool bare = r->xi * r->rc < 0.17;
         const PairScales sc = {r->xi, 2.0 * r->xi / sqrt(3.14159265358979323846),
                                bare ? 1.0 : r->xi, bare};
-        const int bytes = kCap64 * (int)(sizeof(se::d4) + sizeof(se::f4));
+        const int W = 2 * r->K + 1;
+        const double mean = (double)N * W * W * W / r->ncells;   // candidates of a cell
+        const int cap = (int)std::min<double>(kCap64, std::max<double>(kCap64Min, 1.5 * mean));
+        const int each = (int)(sizeof(se::d4) + sizeof(se::f4));
+        // the limit is the kernel's, not the call's: the same for every object
         if (cudaFuncSetAttribute(k_rs_pairs64, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 bytes) != cudaSuccess)
+                                 kCap64 * each) != cudaSuccess)
             return SE_ERR_CUDA;
-        k_rs_pairs64<<<r->ncells, 32 * kPair64Warps, bytes, s>>>(
-            (const V*)r->sorted, r->sorted_f, r->start, r->perm, nc, r->K, L, r->rc * r->rc, rc2_f,
+        k_rs_pairs64<<<r->ncells, 32 * kPair64Warps, cap * each, s>>>(
+            (const V*)r->sorted, r->sorted_f, r->start, r->perm, cap, nc, r->K, L, r->rc * r->rc, rc2_f,
             sc, r->kc, r->table, (T*)phi, (T*)F, acc, r->partials, r->ticket, E);
     } else {
         const int cap = (int)(kNbSmem / sizeof(V));
