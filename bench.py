@@ -381,13 +381,16 @@ def roofline(kind, amount, kernel, us, prec, up, workload_name):
              "peak_source": "152 SMs x 32 shared-memory atomics/clock x max SM clock",
              "probe_peak": up["probe"]["smem_atomic_u32_gops"]}
     elif kind == "flop":
-        fp64 = prec == "fp64"
+        # double precision: the kernels named _fx on split integers, the others
+        # on the FP64 pipe
+        unit = "fp32_fma" if prec != "fp64" else "split_int" if "_fx" in kernel else "fp64_fma"
+        source = {"fp32_fma": "152 SMs x 128 FP32 lanes x 2 flops x max SM clock",
+                  "fp64_fma": "nominal FP64 rate of GB300",
+                  "split_int": "152 SMs x 64 32-bit integer multiply-adds into 64 bits/clock x max "
+                               "SM clock, three for each FP64 multiply-add of 2 flops"}
         r = {"bound": "alu", "unit": "TFLOP/s", "achieved": amount / secs / 1e12,
-             "peak": up["split_int_tflops"] if fp64 else up["fp32_fma_tflops"],
-             "peak_source": ("152 SMs x 64 32-bit integer multiply-adds into 64 bits/clock x max "
-                             "SM clock, three for each FP64 multiply-add of 2 flops" if fp64 else
-                             "152 SMs x 128 FP32 lanes x 2 flops x max SM clock"),
-             "probe_peak": None if fp64 else up["probe"]["fp32_fma_tflops"]}
+             "peak": up[unit + "_tflops"], "peak_source": source[unit],
+             "probe_peak": up["probe"].get(unit + "_tflops")}
     else:
         r = {"bound": "hbm", "unit": "GB/s", "achieved": amount / secs / 1e9,
              "peak": up["hbm_gbs"], "peak_source": up["hbm_source"]}

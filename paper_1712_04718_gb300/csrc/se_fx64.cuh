@@ -227,63 +227,64 @@ k_spread_fx(const int4* __restrict__ fac, const int2* __restrict__ xq,
     if (gi >= GPW) return;
     const int Mp = fp.kp.M + P - 1;
     const int per = (kFxThreads / 32) * GPW;
-    const bool words = grid_bits(acc, fp) > 0;   // uniform over the grid
-    const int ref = (__double2hiint(acc->qunit) >> 20) & 0x7ff;
-    for (long long pl = c0 + (long long)blockIdx.x * per + warp * GPW + gi; pl < c1;
-         pl += (long long)gridDim.x * per) {
-        const int p = (int)pl;
-        const int4 cell = *reinterpret_cast<const int4*>(cells + 4 * (size_t)p);
-        const int4* fy = fac + ((size_t)(p - c0) * 3 + 1) * P;
-        const int2* fx = xq + (size_t)(p - c0) * P;
-        const int2 z = *reinterpret_cast<const int2*>(fy + P + k);
-        unsigned long long* g0 = g64 + ((size_t)cell.x * Mp + cell.y) * Mp + cell.z + k;
-        int shift = 0;
-        if (!words) {
-            split_exponent(sorted[4 * (size_t)p + 3], &shift);
-            shift -= ref + 60;
-        }
-#pragma unroll 1
-        for (int bc = 0; bc < P; bc += BC) {
-            int yzh[BC], yzl[BC];
-#pragma unroll
-            for (int b = 0; b < BC; ++b) {
-                const int2 y = __ldg(reinterpret_cast<const int2*>(fy + bc + b));
-                const long long cr = mad_wide(y.x, z.y, mad_wide(y.y, z.x, 1LL << 29));
-                const long long v = mad_wide(y.x, z.x, cr >> 30);
-                yzh[b] = (int)((v + (1 << 29)) >> 30);
-                yzl[b] = (int)v - (int)((unsigned)yzh[b] << 30);
+    // W: integer sums
+    auto particles = [&](auto W, int ref) {
+        constexpr bool kWords = decltype(W)::value;
+        for (long long pl = c0 + (long long)blockIdx.x * per + warp * GPW + gi; pl < c1;
+             pl += (long long)gridDim.x * per) {
+            const int p = (int)pl;
+            const int4 cell = *reinterpret_cast<const int4*>(cells + 4 * (size_t)p);
+            const int4* fy = fac + ((size_t)(p - c0) * 3 + 1) * P;
+            const int2* fx = xq + (size_t)(p - c0) * P;
+            const int2 z = *reinterpret_cast<const int2*>(fy + P + k);
+            unsigned long long* g0 = g64 + ((size_t)cell.x * Mp + cell.y) * Mp + cell.z + k;
+            int shift = 0;
+            if constexpr (!kWords) {
+                split_exponent(sorted[4 * (size_t)p + 3], &shift);
+                shift -= ref + 60;
             }
-            unsigned long long* ga = g0 + (size_t)bc * Mp;
-            // start: what makes the cuts of the sum round without a preferred sign
-            // (errors of one sign add up over the weights of a cluster)
-            auto planes = [&](long long start, auto add) {
+#pragma unroll 1
+            for (int bc = 0; bc < P; bc += BC) {
+                int yzh[BC], yzl[BC];
+#pragma unroll
+                for (int b = 0; b < BC; ++b) {
+                    const int2 y = __ldg(reinterpret_cast<const int2*>(fy + bc + b));
+                    const long long cr = mad_wide(y.x, z.y, mad_wide(y.y, z.x, 1LL << 29));
+                    const long long v = mad_wide(y.x, z.x, cr >> 30);
+                    yzh[b] = (int)((v + (1 << 29)) >> 30);
+                    yzl[b] = (int)v - (int)((unsigned)yzh[b] << 30);
+                }
+                unsigned long long* ga = g0 + (size_t)bc * Mp;
 #pragma unroll 1
                 for (int a = 0; a < P; ++a, ga += (size_t)Mp * Mp) {
                     const int2 x = __ldg(fx + a);
                     unsigned long long* g = ga;
 #pragma unroll
                     for (int b = 0; b < BC; ++b, g += Mp) {
+                        // the cuts round without a preferred sign (errors of one sign
+                        // add up over the weights of a cluster): integer sums: W cut,
+                        // plus 4, cut by three bits, mean error (-1/2 + 1/2) / 8;
+                        // FP64 sums: W rounded
+                        const long long start = kWords ? 4LL << 30 : 1LL << 29;
                         const long long cr = mad_wide(x.x, yzl[b], mad_wide(x.y, yzh[b], start));
-                        add(g, mad_wide(x.x, yzh[b], (long long)(int)(cr >> 30)));
+                        const long long w = mad_wide(x.x, yzh[b], (long long)(int)(cr >> 30));
+                        if constexpr (kWords) {
+                            atomicAdd(g, (unsigned long long)(w >> 3));
+                        } else {
+                            const double v = __ll2double_rn(w);
+                            const int hi = __double2hiint(v);
+                            if (((hi >> 20) & 0x7ff) + shift > 0)   // not for w = 0: shift <= -60
+                                atomicAdd(reinterpret_cast<double*>(g),
+                                          __hiloint2double(hi + (int)((unsigned)shift << 20),
+                                                           __double2loint(v)));
+                        }
                     }
                 }
-            };
-            if (words) {
-                // W cut, plus 4, cut by three bits: mean error (-1/2 + 1/2) / 8
-                planes(4LL << 30, [](unsigned long long* g, long long w) {
-                    atomicAdd(g, (unsigned long long)(w >> 3));
-                });
-            } else {
-                planes(1LL << 29, [shift](unsigned long long* g, long long w) {
-                    const double v = __ll2double_rn(w);
-                    const int hi = __double2hiint(v);
-                    if (((hi >> 20) & 0x7ff) + shift > 0)   // not for w = 0: shift <= -60
-                        atomicAdd(reinterpret_cast<double*>(g),
-                                  __hiloint2double(hi + (int)((unsigned)shift << 20), __double2loint(v)));
-                });
             }
         }
-    }
+    };
+    if (grid_bits(acc, fp) > 0) particles(std::true_type(), 0);   // uniform over the grid
+    else particles(std::false_type(), (__double2hiint(acc->qunit) >> 20) & 0x7ff);
 }
 
 // A sum of products of split numbers: A + B 2^-30.

@@ -261,19 +261,18 @@ __device__ __forceinline__ df2 warp_sum_partials_df(const float* partials, int n
 
 // Last-block detection: every block stores its partial, fences, and takes a
 // ticket; the block with the last ticket sees all partials.
-__device__ __forceinline__ bool last_block2(unsigned* ticket, unsigned nblocks) {
+__device__ __forceinline__ bool last_block(unsigned* ticket) {
     __shared__ bool is_last;
     __threadfence();
     __syncthreads();
     if (threadIdx.x == 0) {
         unsigned t = atomicAdd(ticket, 1u);
-        is_last = (t == nblocks - 1);
+        is_last = (t == gridDim.x - 1);
     }
     __syncthreads();
     if (is_last) __threadfence();
     return is_last;
 }
-__device__ __forceinline__ bool last_block(unsigned* ticket) { return last_block2(ticket, gridDim.x); }
 
 // Sum of n partials (stride apart, from offset), by the whole block; valid in
 // thread 0.  The loads go through L2 (other blocks wrote them).
@@ -370,9 +369,10 @@ k_bin(const T* __restrict__ xyz, const T* __restrict__ q, const KParams<T> kp,
             acc->nonfinite = (unsigned)s_bad;
             // the scale of the charges: |q| qscale < 1; charges below 2^-1000 keep 2^1000
             const double qmax = __longlong_as_double((long long)sqm);
-            acc->qscale = qmax > 0x1p-1000 ? (1.0 - 0x1p-50) / qmax : 0x1p+1000;
-            acc->qunit = 1.0 / acc->qscale;
-            acc->qmean = (float)(t.y * acc->qscale) / (float)kp.N;
+            const double qs = qmax > 0x1p-1000 ? (1.0 - 0x1p-50) / qmax : 0x1p+1000;
+            acc->qscale = qs;
+            acc->qunit = 1.0 / qs;
+            acc->qmean = __fdividef((float)(t.y * qs), (float)kp.N);
             *ticket = 0u;
         }
     }

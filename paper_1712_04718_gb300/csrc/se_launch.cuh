@@ -57,9 +57,12 @@ template <typename T>
 cudaError_t launch_spread_tiled(const v4_t<T>* sorted, const int* tile_start, T* grid,
                                 const KParams<T>& kp, bool comp, const Acc* acc, cudaStream_t s) {
     switch (kp.P) {
-#define SE_CASE(PP) \
-    case PP: return comp ? spread_tiled_P<T, PP, true>(sorted, tile_start, grid, kp, acc, s) \
-                         : spread_tiled_P<T, PP, false>(sorted, tile_start, grid, kp, acc, s);
+// compensation is a single-precision form
+#define SE_CASE(PP)                                                                    \
+    case PP:                                                                           \
+        if constexpr (std::is_same<T, float>::value)                                   \
+            if (comp) return spread_tiled_P<T, PP, true>(sorted, tile_start, grid, kp, acc, s); \
+        return spread_tiled_P<T, PP, false>(sorted, tile_start, grid, kp, acc, s);
         SE_FOR_EACH_P(SE_CASE)
 #undef SE_CASE
         default: return cudaErrorInvalidValue;

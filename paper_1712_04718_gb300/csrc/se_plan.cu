@@ -1103,6 +1103,7 @@ int se_plan_set_prefactor(se_plan* p, double kc) {
 int se_plan_set_stream(se_plan* p, void* stream) {
     if (!p) return SE_ERR_ARG;
     p->stream = (cudaStream_t)stream;
+    p->fft_stream_set = false;   // a new stream may have an old one's handle
     return SE_OK;
 }
 
