@@ -56,10 +56,16 @@ extern "C" {
 #define SE_ERR_NOMEM (-3)      /* device or host allocation failed */
 #define SE_ERR_UNSUPPORTED (-4)/* valid but not supported: odd P, P > 32 */
 #define SE_ERR_CUFFT (-5)      /* a cuFFT call failed */
-#define SE_ERR_NONFINITE (-6)  /* a position or charge was NaN or infinite */
+#define SE_ERR_NONFINITE (-6)  /* a position or charge was NaN or infinite; the outputs are
+                                  unspecified (NaN charges give NaN, a NaN position may
+                                  count as 0) */
 
 /* precision modes */
-#define SE_FP64 0   /* every step in double precision */
+#define SE_FP64 0   /* every step in double precision.  Sums over a particle's support
+                       run on numbers split into two integers (60 bits of the
+                       largest value); the spread keeps 2^-54 of the mean charge's
+                       largest weight or better and takes FP64 sums where its
+                       integer grid could not (crowded tiles, charges far apart) */
 #define SE_FP32 1   /* single precision with compensated (two-sum) grid
                        accumulation; Green's function table, grid energy and
                        the final energy reduction in double precision */
@@ -96,7 +102,9 @@ int se_plan_set_prefactor(se_plan *plan, double kc);
 int se_plan_set_stream(se_plan *plan, void *stream);
 
 /* Kernel tuning: spread_variant 0 = automatic, 1 = shared-memory tiles and
- * cuFFT, 2 = direct global accumulation and cuFFT (not with SE_FP32),
+ * cuFFT (SE_FP64: global reductions to an integer grid, the default but for few
+ * particles on a large grid; tile then only orders the particles and bounds the
+ * grid's sums), 2 = direct global accumulation and cuFFT (not with SE_FP32),
  * 3 = the single-precision pipeline without cuFFT (SE_FP32 or SE_FP32_PLAIN,
  * M <= 128; the default there): exact 64-bit fixed-point spreading, line DFTs
  * with the scaling fused into the x pass, kernels chained by programmatic

@@ -1,9 +1,9 @@
 // se_fx64.cuh -- double-precision spread and gather (Eq. 3.5, Eq. 3.9 and the
 // analytic force of Sec. 3.1) in integer arithmetic.
 //
-// This GPU retires about 1.6 FP64 operations per clock and SM, but 51
-// multiply-adds of 32-bit integers into 64 bits.  The P^3 sums of a particle
-// therefore run on numbers split into two integers,
+// This GPU retires about 1.7 FP64 operations per clock and SM (the library's own
+// probe; two nominally), but 51 multiply-adds of 32-bit integers into 64 bits.  The
+// P^3 sums of a particle therefore run on numbers split into two integers,
 //     v = hi + lo 2^-30,  hi = round(v), |lo| <= 2^29   (v scaled to at most 2^30),
 // whose product is  hi hi' + (hi lo' + lo hi') 2^-30  with lo lo' (below 2^-60
 // of the largest product) left out: three multiply-adds, exact, and so are
@@ -12,22 +12,24 @@
 //   k_scatter_fx    particles into tile order, and the window factors of each
 //                   (the only FP64 arithmetic per particle: two exponentials,
 //                   a reciprocal and two operations a factor, per dimension)
-//   k_spread_fx     Eq. 3.5: a weight is rounded to a multiple of 2^-56 max|q|
-//                   (grid_bits) and added to a 64-bit integer grid, padded so
-//                   that no support wraps, with global reductions: integer
-//                   sums, the same for every order
-//   k_fx_fold       integer grid -> FP64, its periodic images added
+//   k_spread_fx     Eq. 3.5: a weight is rounded to a multiple of 2^-54 to 2^-56
+//                   max|q| and added to a 64-bit integer grid, padded so that no
+//                   support wraps, with global reductions: integer sums, the same
+//                   for every order.  Where that quantum is too coarse (crowded
+//                   tiles, a few large charges: grid_bits) the weights are added
+//                   as FP64 numbers instead (the last bits then depend on the order)
+//   k_fx_fold       that grid -> FP64, its periodic images added
 //   k_grid_split    the transformed grid split, padded by its periodic images
 //   k_gather_fx     Eq. 3.9 and the forces: y, x and z sums as above, one
 //                   conversion to FP64 per particle and result
 //
 // Measured against FP64 arithmetic (tiles with FP64 shared-memory adds up to P =
 // 12 and global FP64 reductions above for the spread, FP64 sums for the gather),
-// a whole evaluation: 21 642 atoms, M = 52, P = 8: 481 -> 209 us (spread 220 ->
-// 26, gather 136 -> 33); M = 96, P = 24: 2517 -> 1089 us (958 -> 396, 1324 ->
-// 446); 1000 charges, M = 32, P = 16: 181 -> 107 us (53 -> 11, 64 -> 21).  Errors
-// against 64-bit sums 3.3e-14 -> 3.5e-14 (the sums' own), 1.3e-14 -> 2.8e-15 and
-// 1.1e-15 -> 6e-16.
+// a whole evaluation: 21 642 atoms, M = 52, P = 8: 478 -> 201 us (spread 220 ->
+// 25, gather 136 -> 31); M = 96, P = 24: 2517 -> 1074 us (958 -> 382, 1324 ->
+// 405); 1000 charges, M = 32, P = 16: 181 -> 103 us (53 -> 11, 64 -> 18).  Errors of
+// potentials against extended precision 7.1e-15 -> 2.9e-15 (water, P = 8), 1.6e-15
+// -> 3.6e-16 (1000 charges, P = 24), 9.0e-16 -> 3.8e-16 (1000 charges, P = 16).
 //
 // Particles are taken in ranges of the tile order, so that the factors
 // (56 P bytes a particle) never need more than kFxFactorBytes.
@@ -211,7 +213,8 @@ constexpr int kFxThreads = 128;
 //   W = xhi yzhi + (xhi yzlo + xlo yzhi) 2^-30,  |W| < 2^59,
 // an integer in units of 2^-3 of the grid's.  Particles come in tile order, but
 // nothing depends on it.
-// Bound by the L2's 64-bit reductions (about 2.4 lanes per clock and SM).
+// Bound by the reductions: 2.4 lanes per clock and SM at P = 24, with the L1's path
+// to the L2 at 89 % and the L2 at 66 % of their rates (issue 41 %).
 // For FP64 sums (grid_bits) W, an integer of 2^-60 of the particle's own charge,
 // goes as an FP64 number in units of the largest charge's power of two to the
 // same grid, as FP64 reductions.
@@ -316,8 +319,9 @@ __device__ __forceinline__ int2 fx_top(const FxSum& s, int e) {
 // each of the three sums is at most gs times the largest term, gs a bound of
 // the sum of a window's factors; the first two are cut to 32 + e1 and 32 + e2
 // bits less, so that every sum stays below 2^63 (fx_params).
-// Bound by the integer multiply-adds: six of about nine instructions a grid
-// value for potential and force.
+// Bound by latency: six of about nine instructions a grid value are the multiply-
+// adds, but at P = 24 the issue slots are 46 %, the multiply-add pipe 32 % and the
+// L1 52 % busy with 30 warps an SM (128 or 64 registers a thread).
 // Consecutive particles share a block, and with it the L1 cache: up to 512
 // threads (fewer where the particles are too few for every SM).  Supports 14 and
 // 16 keep 16 rows of loads and factors in flight in more than 128 registers

@@ -239,7 +239,7 @@ int fx_tile(se_plan* p) {
     const int n8 = (p->M + 7) / 8;
     int best = 8;
     double least = 0.0;
-    if (p->N <= (int64_t)16 * n8 * n8 * n8) return best;
+    if (p->M > 140 || p->N <= (int64_t)16 * n8 * n8 * n8) return best;
     for (int t = 8; t >= 4; --t) {
         if (20 * t < p->M && t < 8) break;
         p->tile = std::min(t, p->M);

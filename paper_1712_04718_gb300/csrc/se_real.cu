@@ -430,9 +430,10 @@ k_rs_pairs(const se::f4* __restrict__ sorted, const int* __restrict__ start,
 }
 
 // ---------------------------------------------------------------------------
-// Double precision.  This GPU retires about two FP64 operations per clock and
-// SM, a 64th of its FP32 rate, so the kernel is bound by the FP64 operations
-// of its pairs and by nothing else; the design spends as few as it can:
+// Double precision.  This GPU retires about 1.7 FP64 operations per clock and SM
+// (the library's own probe; two nominally, a 64th of its FP32 rate), so the kernel
+// is bound by the FP64 operations of its pairs and by nothing else (its FP64 pipe
+// is 84 % busy); the design spends as few as it can:
 //
 //  - The distance test, which 73 % of the candidates fail on a water box, is
 //    made in FP32, on positions in units of L, with a bound wide enough for
@@ -450,8 +451,8 @@ k_rs_pairs(const se::f4* __restrict__ sorted, const int* __restrict__ start,
 // are evaluated by the 32 lanes, so that all lanes of the FP64 pipe work.
 //
 // 21 642-atom water box, r_c = 1 nm (420 pairs a particle): 3314 -> 626 us a
-// call, of which the 27 operations of its 9.1 M pairs take 390 us at the
-// pipe's rate; the error against 64-bit sums 8.3e-16 -> 8.1e-16.
+// call, of which the 27 operations of its 9.1 M pairs take 470 us at the
+// probed rate; the error against 64-bit sums 8.3e-16 -> 8.1e-16.
 constexpr int kVMinExp = -5, kVMaxExp = 6;   // the table covers 2^-5 <= v < 2^6
 constexpr int kVDeg = 7;
 // rows per octave: 64 below v = 16, then 128 and 256 (e^{-v} needs shorter
@@ -494,7 +495,7 @@ struct PairScales {
 
 constexpr int kPair64Warps = 6;
 // Staged candidates: at most 2048 (96 KB: two CTAs per SM); half a box's mean count
-// over, and at least 512 (24 KB: five CTAs, as many as the registers allow), where
+// over, and at least 512 (24 KB: four CTAs, as many as the registers allow), where
 // fewer will do (rs_run): sparse cells are many short CTAs (20 000 particles in
 // 40^3 cells: 780 us at 2048, 548 at 512; with FP64 arithmetic for every pair 755).
 constexpr int kCap64 = 2048, kCap64Min = 512;

@@ -1,12 +1,12 @@
-"""The double-precision spread and gather (integer and FP32 arithmetic on split
-numbers) where they can go wrong: every support, tile edges with constant and
-with run-time row strides, several x-slabs a tile, more particles a tile than
-one round of the integer words takes, few particles, charges far from one,
-flat windows (the gather's scales), several ranges of particles, and input
-beyond the range or not finite.
+"""The double-precision spread and gather (integer arithmetic on split numbers)
+where they can go wrong: every support, tile edges that do and do not divide the
+grid, tiles and cells with more particles than the integer grid has bits for,
+few particles, charges far from one, flat windows (the gather's scales), several
+ranges of particles, and input beyond the range or not finite.
 
 Tolerances as the other FP64 comparisons: 1e-12 for the grid (weights are
-multiples of 2^-52 of the largest charge's), 5e-12 for particle outputs."""
+multiples of 2^-54 or less of the largest charge's, or FP64 numbers), 5e-12 for
+particle outputs."""
 import math
 
 import numpy as np
